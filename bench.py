@@ -49,7 +49,8 @@ FP32_LANES_PER_SM = 128
 WORKLOAD = "dq-julia 1920x1080, c~U[-0.8,0.8]^8 seeds 0-4, max_iter 16, 512 march + 10 bisect"
 MODE_NAMES = {0: "FP32", 1: "FP32 + FP64 recheck (margin 1e-3)", 2: "FP64"}
 DTYPES = {0: "f32", 1: "f32+f64-recheck", 2: "f64"}
-KERNEL_SOURCES = ("paper_2303_14827_gb300/csrc/render.cu", "paper_2303_14827_gb300/csrc/render_common.cuh",
+KERNEL_SOURCES = ("paper_2303_14827_gb300/csrc/render_passes.cuh", "paper_2303_14827_gb300/csrc/settle.cuh",
+                  "paper_2303_14827_gb300/csrc/render_common.cuh",
                   "paper_2303_14827_gb300/csrc/dq_math.cuh", "paper_2303_14827_gb300/csrc/dqj_internal.h")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "march4_kernel_1080p.md")
 

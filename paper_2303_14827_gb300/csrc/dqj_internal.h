@@ -79,7 +79,12 @@ struct alignas(16) FrameDesc {
     int32_t k_chunk;      // samples per range
     int32_t tile_part;    // the frame's tiles t with t mod tile_parts == tile_part are rendered
     int32_t tile_parts;   // (1: every tile)
-    int32_t march_samples;  // paired FP32 march on an axis-aligned slice: samples of each ray per round (1, 2)
+    int32_t march_samples;  // paired FP32 march: samples of each ray per round (1, 2)
+    // settled blocks (settle.cuh): thresholds of a proved escape and of a proved
+    // bounded step (R^2 and the recheck margin, with room for rounding), |c|,
+    // |slice origin| + |eye|, and whether blocks are settled (march_settles)
+    float settle_hi, settle_lo, settle_cn, settle_an;
+    int32_t settle;
 };
 
 // Counters at the head of the scratch block; zeroed before every frame.
@@ -112,11 +117,13 @@ struct alignas(16) Scratch {
     uint32_t pad_[3];
 };
 
-// Host-side launch helpers implemented in render.cu.
+// Host-side launch helpers (render.cu).
 // Enqueue the passes of one frame on st.  ev (optional, 5 events) is recorded
 // before the march and after the march, bisect, recheck and fixup passes.
 cudaError_t launch_frame(const FrameDesc &fd, const Scratch &sc, cudaStream_t st, int num_sms,
                          cudaEvent_t *ev = nullptr);
+// launch_frame for the march with the component-wise square (render_componentwise.cu).
+cudaError_t launch_componentwise(const FrameDesc &fd, const Scratch &sc, cudaStream_t st, int num_sms, cudaEvent_t *ev);
 // The distance-estimate traversal (de.cu): sphere tracing, then normal and
 // shading of its hits; same events (the last three after the shading pass).
 cudaError_t launch_de(const FrameDesc &fd, const Scratch &sc, cudaStream_t st, int num_sms, cudaEvent_t *ev);
@@ -124,9 +131,12 @@ cudaError_t fma_peak_launch(int variant, int num_sms, float *sink, cudaStream_t 
 // Ranges the paired FP32 march of a frame splits its samples into (1: none):
 // enough for the frame's tiles to fill the resident warps of num_sms SMs.
 int march_split(const FrameDesc &fd, int num_sms);
-// Samples of each ray per round of the paired FP32 march on an axis-aligned
-// slice: 2 unless DQJ_MARCH_SAMPLES = 1 (read once per process).  Both give
-// the same results.
+// Form of the march, from DQJ_MARCH_SAMPLES (read once per process): samples of
+// each ray per round of the paired FP32 kernel, 2 unless the variable is 1, and
+// whether blocks of samples are settled by a bound (settle.cuh), in every
+// precision: yes unless the variable is 0 (two per round, every sample marched)
+// or 1.  All forms give the same results.
 int march_samples_per_round();
+bool march_settles();
 
 }  // namespace dqj

@@ -7,6 +7,7 @@
 #include <atomic>
 
 #include "dq_math.cuh"
+#include "settle.cuh"
 
 namespace dqj {
 
@@ -693,9 +694,14 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
 // sample k + 1 after an inside sample k is classified but not counted or
 // staged, as the one-sample march never reaches it.  SPLIT: samples [kb, ke)
 // of each ray with the range's partial result, as in march2_tile.
-template <int SQ, int MOD, bool RECHECK, bool AXIS = true, bool SPLIT = false>
+// The tile's samples are taken 512 at a time: blocks of them whose escape
+// count a bound proves (settle_chunk) only add to the counts, the rounds of
+// the others are marched in order.  Without SETTLE all of them are (a split
+// march's ranges and frames of few, wide samples do not pay for the bound, and
+// the loop without it is the shorter one).  box: the warp's, in shared memory.
+template <int SQ, int MOD, bool RECHECK, bool AXIS, bool SPLIT, bool SETTLE>
 __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConsts &P, const Scratch &sc, unsigned tile,
-                                            LaneStats &st, int4 *qs = nullptr, int kb = 0, int ke = 0)
+                                            LaneStats &st, TileBox &box, int4 *qs = nullptr, int kb = 0, int ke = 0)
 {
     const FrameT<float> &F = fd.f;
     const int lane = threadIdx.x & 31;
@@ -729,6 +735,7 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
         }
         if (!acta) tia = toa = 0.f;
         if (!actb) tib = tob = 0.f;
+        if (SETTLE && fd.settle) tile_box(fd, acta, da, tia, toa, actb, db, tib, tob, box);
         dl = make_float2((toa - tia) / (float)N, (tob - tib) / (float)N);
         if (RECHECK) {  // a half without a ray samples far away: never within the recheck band
             if (!acta) tia = kFarT;
@@ -758,14 +765,50 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     int suma = 0, sumb = 0, maxa = 0, maxb = 0, kfa = -1, kfb = -1;
     int qn = 0;  // staged recheck entries (warp-uniform)
     const int k0 = SPLIT ? kb : 0, k1 = SPLIT ? ke : N + 1;
-    float2 kf = make_float2((float)k0, (float)k0);
-    const float2 one = make_float2(1.f, 1.f), two = make_float2(2.f, 2.f), far = make_float2(kFarT, kFarT);
+    const float2 far = make_float2(kFarT, kFarT);
     bool more = __any_sync(kFull, acta || actb);
-    for (int k = k0; k < k1 && more; k += 2) {
+    // settled samples: the chunk [kc, kce) in hand, its
+    // words of settled counts, the blocks and pairs of it still to march
+    const bool settle = SETTLE && fd.settle && k1 > kSettleMin;
+    int kc = k0 - kSettleChunk, kce = kc, pairs = 1, b = 0, p = 0;
+    unsigned w = 0, open = 0, blocks = 0, ob = 0;
+    float kf = (float)k0;  // k, carried along: a conversion would head every round's chain
+    for (int k = k0; more; k += 2, kf += 2.f) {
+        if (settle) {
+            while (!ob) {
+                if (!blocks) {  // the chunk is through: its settled samples, then the next chunk
+                    if (kce > k0) {
+                        int s, m;
+                        settled_before(w, kc, kce, pairs, 32, 0, s, m);
+                        suma += acta ? s : 0;
+                        sumb += actb ? s : 0;
+                        maxa = max(maxa, acta ? m : 0);
+                        maxb = max(maxb, actb ? m : 0);
+                    }
+                    kc += kSettleChunk;
+                    if (kc >= k1) break;
+                    kce = min(kc + kSettleChunk, k1);
+                    pairs = settle_pairs(kce - kc);
+                    w = kce - kc > kSettleMin ? settle_chunk<SQ, MOD, AXIS>(fd, box, kc, kce, pairs) : 0u;
+                    open = open_pairs(w, kc, kce, pairs);
+                    blocks = __ballot_sync(kFull, open != 0);
+                    continue;
+                }
+                b = __ffs(blocks) - 1;
+                blocks &= blocks - 1;
+                ob = __shfl_sync(kFull, open, b);
+            }
+            if (!ob) break;  // no chunk is left
+            p = (__ffs(ob) - 1) >> 2;
+            ob &= ob - 1;
+            k = kc + 2 * (pairs * b + p);
+            kf = (float)k;
+        }
+        if (k >= k1) break;
         const bool has2 = k + 1 < k1;  // warp-uniform: an odd number of samples ends in a round of one
-        const float2 t = f2fma(kf, dl, tin);
-        const float2 t2 = has2 ? f2fma(f2add(kf, one), dl, tin) : far;
-        kf = f2add(kf, two);
+        const float kf2 = kf + 1.f;
+        const float2 t = f2fma(make_float2(kf, kf), dl, tin);
+        const float2 t2 = has2 ? f2fma(make_float2(kf2, kf2), dl, tin) : far;
         float2 z[8], y[8];
         bool ina = acta, inb = actb, ina2 = acta && has2, inb2 = actb && has2, live;
         int ca, cb, ca2, cb2;
@@ -826,6 +869,18 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
             if (RECHECK) {  // a finished ray samples far away from now on (see above)
                 if (da) tin.x = kFarT;
                 if (db) tin.y = kFarT;
+            }
+            if (settle) {  // rays that end here: their settled samples of this chunk so far
+                int s, m;
+                settled_before(w, kc, kce, pairs, b, p, s, m);
+                if (da) {
+                    suma += s;
+                    maxa = max(maxa, m);
+                }
+                if (db) {
+                    sumb += s;
+                    maxb = max(maxb, m);
+                }
             }
             acta = acta && !da;
             actb = actb && !db;

@@ -149,10 +149,11 @@ __device__ __forceinline__ Scratch load_scratch(const Scratch *src)
 // dqj_render takes (fd.march_samples), so a served request's counters equal
 // those of the alone render.
 template <bool RECHECK, bool AXIS>
-__device__ __noinline__ void march_item4(const FrameDesc &fd, const Scratch &sc, unsigned tile, int4 *stage)
+__device__ __noinline__ void march_item4(const FrameDesc &fd, const Scratch &sc, unsigned tile, TileBox &box,
+                                         int4 *stage)
 {
     LaneStats st;
-    march4_tile<0, 0, RECHECK, AXIS>(fd, fd.p2, sc, tile, st, stage);
+    march4_tile<0, 0, RECHECK, AXIS, false, true>(fd, fd.p2, sc, tile, st, box, stage);
     flush_lane_stats<false>(sc, st, true);
 }
 
@@ -165,10 +166,11 @@ __device__ __noinline__ void march_item2(const FrameDesc &fd, const Scratch &sc,
 }
 
 template <bool RECHECK, bool AXIS>
-__device__ __forceinline__ void march_item(const FrameDesc &fd, const Scratch &sc, unsigned tile, int4 *stage)
+__device__ __forceinline__ void march_item(const FrameDesc &fd, const Scratch &sc, unsigned tile, TileBox &box,
+                                           int4 *stage)
 {
     if (fd.march_samples == 2)
-        march_item4<RECHECK, AXIS>(fd, sc, tile, stage);
+        march_item4<RECHECK, AXIS>(fd, sc, tile, box, stage);
     else
         march_item2<RECHECK, AXIS>(fd, sc, tile, stage);
 }
@@ -207,6 +209,7 @@ __device__ __forceinline__ unsigned claim(unsigned long long *ctr, unsigned tota
 __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
 {
     __shared__ FrameDesc s_fd[kBlock / 32];
+    __shared__ TileBox s_box[kBlock / 32];
     __shared__ int4 s_stage[kBlock / 32][kQStage];  // recheck entries of a march tile, per warp
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
@@ -290,14 +293,14 @@ __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
         if (ph == kPhaseMarch) {
             if (recheck) {
                 if (fd.axis_slice)
-                    march_item<true, true>(fd, sc, item, s_stage[wib]);
+                    march_item<true, true>(fd, sc, item, s_box[wib], s_stage[wib]);
                 else
-                    march_item<true, false>(fd, sc, item, s_stage[wib]);
+                    march_item<true, false>(fd, sc, item, s_box[wib], s_stage[wib]);
             } else {
                 if (fd.axis_slice)
-                    march_item<false, true>(fd, sc, item, nullptr);
+                    march_item<false, true>(fd, sc, item, s_box[wib], nullptr);
                 else
-                    march_item<false, false>(fd, sc, item, nullptr);
+                    march_item<false, false>(fd, sc, item, s_box[wib], nullptr);
             }
             done_ctr = &b->tile_done;
             n_items = 1;
