@@ -85,6 +85,7 @@ struct alignas(16) FrameDesc {
     // |slice origin| + |eye|, and whether blocks are settled (march_settles)
     float settle_hi, settle_lo, settle_cn, settle_an;
     int32_t settle;
+    double inv_n;     // 1 / N
 };
 
 // Counters at the head of the scratch block; zeroed before every frame.

@@ -109,48 +109,6 @@ __device__ __forceinline__ bool camera_clip(const FrameT<T> &F, int W, int H, in
     return ok && (t0 < t1);
 }
 
-// FP64 camera ray and box clip for the recheck of a queued sample: the
-// quantities of camera_clip<double> with the pixel-to-screen map folded into one
-// FMA per axis and reciprocals in place of divisions (far fewer FP64
-// instructions; FP64 runs at 1/64 of the FP32 rate).  Each value may differ from the reference formula's in the
-// last place, as the FP64 iteration's contracted FMAs already do: far below
-// what moves a recheck decision, which is taken against a margin of 1e-3
-// relative.
-__device__ __forceinline__ bool camera_clip_rcp(const FrameT<double> &F, int x, int y, double (&d)[3],
-                                                double &t_in, double &t_out)
-{
-    const double sx = fma(double(x) + 0.5, F.sxa, F.sxb);
-    const double sy = fma(double(y) + 0.5, F.sya, F.syb);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) d[a] = F.fwd[a] + sx * F.right[a] + sy * F.upv[a];
-    const double il = rsqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) d[a] = d[a] * il;
-    double t0 = -tinf<double>(), t1 = tinf<double>();
-    bool ok = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        if (d[a] == 0.0) {
-            if (F.eye[a] < F.bmin[a] || F.eye[a] > F.bmax[a]) ok = false;
-        } else {
-            const double inv = __drcp_rn(d[a]);
-            double ta = (F.bmin[a] - F.eye[a]) * inv;
-            double tb = (F.bmax[a] - F.eye[a]) * inv;
-            if (ta > tb) {
-                const double tmp = ta;
-                ta = tb;
-                tb = tmp;
-            }
-            t0 = ta > t0 ? ta : t0;
-            t1 = tb < t1 ? tb : t1;
-        }
-    }
-    if (t0 < 0.0) t0 = 0.0;
-    t_in = t0;
-    t_out = t1;
-    return ok && (t0 < t1);
-}
-
 // D = E d: direction of the ray in the 8-D slice.
 template <typename T>
 __device__ __forceinline__ void slice_dir(const FrameT<T> &F, const T (&d)[3], T (&D)[8])
@@ -278,25 +236,78 @@ __device__ __forceinline__ void shade_write(const FrameDesc &fd, const FrameT<T>
             make_uchar4(to_u8(v * F.albedo[0]), to_u8(v * F.albedo[1]), to_u8(v * F.albedo[2]), 255);
 }
 
+// A pixel's camera ray eye + tau w, not normalised (a sample's position depends
+// only on its fraction of the ray's part inside the box).
+template <typename T>
+__device__ __forceinline__ void ray_w(const FrameT<T> &F, int x, int y, T (&w)[3])
+{
+    const T sx = dfma(T(x) + T(0.5), F.sxa, F.sxb), sy = dfma(T(y) + T(0.5), F.sya, F.syb);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) w[a] = dfma(sy, F.upv[a], dfma(sx, F.right[a], F.fwd[a]));
+}
+
+// FP64 entry and exit (tau) of a ray that crosses the box.  Only the faces that
+// can decide (within 1e-4 of the farthest entry or the nearest exit in FP32)
+// are intersected in FP64: one or two of three, and each needs one reciprocal,
+// formed by two Newton steps on an FP32 one (relative error 1e-7, 1e-14, then
+// rounding).  FP64 runs at 1/64 of the FP32 rate here: with the normalised
+// direction, three reciprocals and the whole clip a recheck took about 130 FP64
+// instructions, in this form about 85.
+__device__ __forceinline__ void ray_clip64(const FrameDesc &fd, const double (&w)[3], double &t0, double &t1)
+{
+    const FrameT<float> &f = fd.f;
+    const FrameT<double> &F = fd.d;
+    float rw[3], in = 0.f, out = tinf<float>(), near[3], far[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float wf = (float)w[a];
+        const bool flat = !(fabsf(wf) > 1e-30f);  // parallel to the slab, inside it
+        rw[a] = 1.f / wf;
+        const float p = (f.bmin[a] - f.eye[a]) * rw[a], q = (f.bmax[a] - f.eye[a]) * rw[a];
+        near[a] = flat ? -tinf<float>() : fminf(p, q);
+        far[a] = flat ? tinf<float>() : fmaxf(p, q);
+        in = fmaxf(in, near[a]);
+        out = fminf(out, far[a]);
+    }
+    t0 = 0.0;
+    t1 = tinf<double>();
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const bool ci = near[a] >= in - 1e-4f * in, co = far[a] <= out + 1e-4f * fabsf(out);
+        if (ci || co) {
+            double r = (double)rw[a];
+            r = fma(r, fma(-w[a], r, 1.0), r);
+            r = fma(r, fma(-w[a], r, 1.0), r);
+            const bool up = rw[a] > 0.f;
+            if (ci) t0 = fmax(t0, ((up ? F.bmin[a] : F.bmax[a]) - F.eye[a]) * r);
+            if (co) t1 = fmin(t1, ((up ? F.bmax[a] : F.bmin[a]) - F.eye[a]) * r);
+        }
+    }
+}
+
 // FP64 recheck of one queued sample {pixel, k | b << 16, path, n32}: the sample
-// is recomputed from the FP64 camera ray with the oracle's formulas (a march
-// sample t_in + k delta, or bisection level b of the bracket (k - 1, k) replayed
-// from the path bits), classified in FP64, and the pixel is queued for an FP64
-// re-render when its FP64 escape count differs from the FP32 one.
+// is placed on its FP64 ray (a march sample k, with x | y << 16 in place of the
+// path, or bisection level b of the bracket (k - 1, k) replayed from the path
+// bits), classified in FP64, and the pixel is queued for an FP64 re-render when
+// its FP64 escape count differs from the FP32 one.  Positions may differ from
+// the reference formula's in the last place, as the FP64 iteration's contracted
+// FMAs already do.
 template <int SQ, int MOD>
 __device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch &sc, int4 e)
 {
     const FrameT<double> &F = fd.d;
     const int pixel = e.x, k = e.y & 0xffff, b = e.y >> 16;
-    const int x = pixel % fd.W, y = pixel / fd.W;
-    double d[3], t_in, t_out;
-    camera_clip_rcp(F, x, y, d, t_in, t_out);
-    const double delta = (t_out - t_in) / (double)fd.N;
+    const bool march = b == kMarchSample;
+    const int x = march ? e.z & 0xffff : pixel % fd.W, y = march ? e.z >> 16 : pixel / fd.W;
+    double w[3], t_in, t_out;
+    ray_w<double>(F, x, y, w);
+    ray_clip64(fd, w, t_in, t_out);
+    const double delta = (t_out - t_in) * fd.inv_n;
     double t;
-    if (b == kMarchSample) {
-        t = t_in + (double)k * delta;
+    if (march) {
+        t = fma((double)k, delta, t_in);
     } else {
-        double lo = t_in + (double)(k - 1) * delta, hi = t_in + (double)k * delta;
+        double lo = fma((double)(k - 1), delta, t_in), hi = fma((double)k, delta, t_in);
         for (int l = 0; l < b; ++l) {
             const double mid = lo + 0.5 * (hi - lo);
             if ((unsigned)e.z >> l & 1u)
@@ -309,21 +320,18 @@ __device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch
     double z[8];
     int n64;
     if (fd.axis_slice) {
-        // components 3..7 of the slice point are zero (the general sum below
-        // gives +-0 there), so the first step takes the axis form, whose
-        // operations are those of dq_iter on those zeros: the same iterate
+        // components 3..7 of the slice point are zero, so the first step takes
+        // the axis form, whose operations are those of dq_iter on those zeros
 #pragma unroll
         for (int j = 0; j < 3; ++j)
-            z[j] = F.O[j] + (F.eye[0] + t * d[0]) * F.E[0][j] + (F.eye[1] + t * d[1]) * F.E[1][j] +
-                   (F.eye[2] + t * d[2]) * F.E[2][j];
+            z[j] = fma(t, fma(w[0], F.E[0][j], fma(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
 #pragma unroll
         for (int j = 3; j < 8; ++j) z[j] = 0.0;
         n64 = classify_scalar_axis<double, SQ, MOD>(z, F, fd.max_iter);
     } else {
 #pragma unroll
         for (int j = 0; j < 8; ++j)
-            z[j] = F.O[j] + (F.eye[0] + t * d[0]) * F.E[0][j] + (F.eye[1] + t * d[1]) * F.E[1][j] +
-                   (F.eye[2] + t * d[2]) * F.E[2][j];
+            z[j] = fma(t, fma(w[0], F.E[0][j], fma(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
         n64 = classify_scalar<double, SQ, MOD>(z, F, fd.max_iter);
     }
     if (n64 != e.w) mark_dirty(fd, sc, pixel);
@@ -547,7 +555,7 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
     // live across the march loop (the recheck mode keeps the linear indices)
     auto px = [&](int slot) { return tx * fd.tile_w + slot % fd.tile_w; };
     auto py = [&](int slot) { return ty * fd.tile_h + slot / fd.tile_w; };
-    int pixa = 0, pixb = 0;
+    int pixa = 0, pixb = 0, xya = 0, xyb = 0;
     bool acta, actb, skipa = false, skipb = false;
     // Axis-aligned slice: zeta_0 = A + t D (components 0..2).  Otherwise the
     // first-iterate form (first_iterate_coeffs): zeta_1 = Q0 + s (Q1 + s Q2),
@@ -559,6 +567,8 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
         if (RECHECK) {
             pixa = ya * fd.W + xa;
             pixb = yb * fd.W + xb;
+            xya = xa | (ya << 16);
+            xyb = xb | (yb << 16);
         }
         const bool va = xa < fd.W && ya < fd.H, vb = xb < fd.W && yb < fd.H;
         float da[3] = {0.f, 0.f, 1.f}, db[3] = {0.f, 0.f, 1.f};
@@ -629,8 +639,8 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
             const unsigned ba = __ballot_sync(kFull, pa), bb = __ballot_sync(kFull, pb);
             const unsigned below = (1u << lane) - 1u;
             const int nqa = __popc(ba), nq = nqa + __popc(bb);
-            if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k | (kMarchSample << 16), 0, ina ? 0 : ca + 1);
-            if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), 0, inb ? 0 : cb + 1);
+            if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k | (kMarchSample << 16), xya, ina ? 0 : ca + 1);
+            if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), xyb, inb ? 0 : cb + 1);
             qn += nq;
             if (qn > kQStage - 64) {
                 flush_staged(fd, sc, qs, qn);
@@ -709,7 +719,7 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     const int tx = (int)(tile % (unsigned)fd.tiles_x), ty = (int)(tile / (unsigned)fd.tiles_x);
     auto px = [&](int slot) { return tx * fd.tile_w + slot % fd.tile_w; };
     auto py = [&](int slot) { return ty * fd.tile_h + slot / fd.tile_w; };
-    int pixa = 0, pixb = 0;
+    int pixa = 0, pixb = 0, xya = 0, xyb = 0;
     bool acta, actb, skipa = false, skipb = false;
     // as in march2_tile: zeta_0 = A + t D on an axis slice, else the first
     // iterate Q0 + s (Q1 + s Q2) with Q0 in D and s = t + dot
@@ -720,6 +730,8 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
         if (RECHECK) {
             pixa = ya * fd.W + xa;
             pixb = yb * fd.W + xb;
+            xya = xa | (ya << 16);
+            xyb = xb | (yb << 16);
         }
         const bool va = xa < fd.W && ya < fd.H, vb = xb < fd.W && yb < fd.H;
         float da[3] = {0.f, 0.f, 1.f}, db[3] = {0.f, 0.f, 1.f};
@@ -834,8 +846,8 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
                 const bool pa = acta && dm.x <= P.margin_t, pb = actb && dm.y <= P.margin_t;
                 const unsigned ba = __ballot_sync(kFull, pa), bb = __ballot_sync(kFull, pb);
                 const int nqa = __popc(ba);
-                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k | (kMarchSample << 16), 0, ina ? 0 : ca + 1);
-                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), 0, inb ? 0 : cb + 1);
+                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k | (kMarchSample << 16), xya, ina ? 0 : ca + 1);
+                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), xyb, inb ? 0 : cb + 1);
                 qn += nqa + __popc(bb);
                 if (qn > kQStage - 64) {
                     flush_staged(fd, sc, qs, qn);
@@ -848,8 +860,8 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
                 const unsigned ba = __ballot_sync(kFull, pa), bb = __ballot_sync(kFull, pb);
                 const int nqa = __popc(ba);
                 const int k2 = k + 1;
-                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k2 | (kMarchSample << 16), 0, ina2 ? 0 : ca2 + 1);
-                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k2 | (kMarchSample << 16), 0, inb2 ? 0 : cb2 + 1);
+                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k2 | (kMarchSample << 16), xya, ina2 ? 0 : ca2 + 1);
+                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k2 | (kMarchSample << 16), xyb, inb2 ? 0 : cb2 + 1);
                 qn += nqa + __popc(bb);
                 if (qn > kQStage - 64) {
                     flush_staged(fd, sc, qs, qn);

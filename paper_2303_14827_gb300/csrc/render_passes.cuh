@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kBlock) march_kernel(const __grid_constant__ F
             }
             if (RECHECK) {
                 const bool push = active && mg;
-                if (warp_push(push, make_int4(y * fd.W + x, k | (kMarchSample << 16), 0, n), sc.queue,
+                if (warp_push(push, make_int4(y * fd.W + x, k | (kMarchSample << 16), x | (y << 16), n), sc.queue,
                               sc.queue_cap, &sc.ctr->queue_count)) {
                     atomicAdd(&sc.ctr->stats[7], 1ull);
                     mark_dirty(fd, sc, y * fd.W + x);

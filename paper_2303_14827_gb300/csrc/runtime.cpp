@@ -293,6 +293,7 @@ void derive_frame(const dqj_params &p, FrameDesc &fd, int tile_w, int tile_h)
     F.de_scale = p.de_step_scale;
     F.de_rb = p.de_bound_radius;
     cast_frame<float>(F, fd.f);
+    fd.inv_n = 1.0 / (double)p.march_steps;
     for (int i = 0; i < 8; ++i) {
         fd.p2.c[i] = make_float2(fd.f.c[i], fd.f.c[i]);
         fd.p2.A[i] = make_float2(fd.f.A[i], fd.f.A[i]);
