@@ -337,6 +337,98 @@ __device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch
     if (n64 != e.w) mark_dirty(fd, sc, pixel);
 }
 
+// Is the FP32 escape count n32 of march sample k of pixel (x, y) certain?  The
+// sample's FP32 orbit is run again beside a bound of its distance from the exact
+// orbit, (er, ed) on the real and dual halves: the rounding of the sample's
+// position, then per step
+//     er <- 2 |z_r| er + er^2 + rounding,  ed <- 2 (|z_r| ed + |z_d| er + er ed) + rounding
+// (algebraic square; quaternion norms multiply), so a step's exact modulus lies
+// within 2 (|z_r| er + |z_d| ed) + er^2 + ed^2 of the FP32 one.  Where every
+// step up to n32 decides clear of that, FP64 can only give n32 too, and the
+// sample needs no FP64 evaluation.  A sample is flagged within 1e-3 of R^2
+// (by default); after the one to three steps of most flagged samples the bound
+// is 1e-5 to 1e-4 of it.
+//
+// Rounding, with u = 2^-24: the camera map's constants and three FMAs put w
+// within 8 u m of the exact direction, m = |fwd| + |sx| + |sy| a bound of its
+// terms; a face parameter tau = (face - eye) / w then lies within
+// |tau| (8 u m / |w_a| + 8 u) + 3 u (|face| + |eye|) / |w_a| of its exact
+// value, and the entry (a maximum) and
+// exit (a minimum) within what the faces' upper and lower values give; the
+// position A + tau W adds 4 u of its terms.  A step's FMAs, each rounding at
+// most u of a term bounded by |z|^2 + |c|, err by less than 16 u of that.
+template <int SQ, int MOD, bool AXIS>
+__device__ __forceinline__ bool count_certain(const FrameDesc &fd, int x, int y, int k, int n32)
+{
+    const FrameT<float> &F = fd.f;
+    constexpr float u = 5.9604645e-8f;
+    float z[8], er, ed;
+    {
+        float w[3];
+        ray_w<float>(F, x, y, w);
+        const float sx = fmaf((float)x + 0.5f, F.sxa, F.sxb), sy = fmaf((float)y + 0.5f, F.sya, F.syb);
+        // terms of sx and sy: up to twice their largest magnitude over the frame
+        const float m = 1.f + fabsf(sx) + fabsf(sy) + 2.f * (fabsf(F.sxb) + fabsf(F.syb));
+        const float dw = 8.f * u * m;
+        float in = 0.f, in_hi = 0.f, in_lo = 0.f, out = tinf<float>(), out_hi = tinf<float>(), out_lo = tinf<float>();
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const float r = 1.f / w[a];
+            const float p = (F.bmin[a] - F.eye[a]) * r, q = (F.bmax[a] - F.eye[a]) * r;
+            const float near = fminf(p, q), far = fmaxf(p, q), rel = fmaf(dw, fabsf(r), 8.f * u);
+            // the faces and the eye are rounded, and their difference may cancel
+            const float abs_r = 3.f * u * fabsf(r) * (fabsf(F.eye[a]) + fmaxf(fabsf(F.bmin[a]), fabsf(F.bmax[a])));
+            const float dn = fmaf(rel, fabsf(near), abs_r), df = fmaf(rel, fabsf(far), abs_r);
+            in = fmaxf(in, near);
+            in_hi = fmaxf(in_hi, near + dn);
+            in_lo = fmaxf(in_lo, near - dn);
+            out = fminf(out, far);
+            out_hi = fminf(out_hi, far + df);
+            out_lo = fminf(out_lo, far - df);
+        }
+        const float tau = fmaf((float)k * (float)fd.inv_n, out - in, in);
+        const float dtau = fmaxf(fmaxf(in_hi - in, in - in_lo), fmaxf(out_hi - out, out - out_lo)) + 8.f * u * out;
+        const float wn = sqrt_approx(fmaf(w[2], w[2], fmaf(w[1], w[1], w[0] * w[0])));
+        // |A| <= settle_an; three FMAs per component of W, one of the position
+        er = 1.01f * fmaf(dtau, wn, fmaf(out, dw, 8.f * u * fmaf(out, wn, fd.settle_an)));
+        if (!(er < 1e-3f)) return false;  // far camera, grazing ray, overflow: FP64 decides
+        ed = AXIS ? 0.f : er;
+#pragma unroll
+        for (int j = 0; j < (AXIS ? 3 : 8); ++j)
+            z[j] = fmaf(tau, fmaf(w[0], F.E[0][j], fmaf(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
+        if (AXIS) {
+#pragma unroll
+            for (int j = 3; j < 8; ++j) z[j] = 0.f;
+        }
+    }
+    float sp = dq_sp<float>(z), m = 0.f;
+    float r2 = fmaf(z[0], z[0], sp), d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
+    const int last = n32 ? n32 : fd.max_iter;
+    for (int n = 1; n <= last; ++n) {
+        const float ar = sqrt_approx(r2), ad = sqrt_approx(d2);
+        const float round = 16.f * u * (r2 + d2 + fd.settle_cn);
+        const float ner = fmaf(er, fmaf(2.f, ar, er), round);
+        if (SQ == 0)
+            ed = fmaf(2.f, fmaf(ar, ed, fmaf(ad, er, er * ed)), round);
+        else
+            ed = fmaf(ed, fmaf(2.f, ad, ed), round);
+        er = ner;
+        dq_iter<float, SQ, MOD>(z, z, sp, F.c);
+        r2 = fmaf(z[0], z[0], sp);
+        d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
+        m = MOD == 0 ? r2 + d2 : r2;
+        const float br = sqrt_approx(r2), bd = MOD == 0 ? sqrt_approx(d2) : 0.f, e2 = MOD == 0 ? ed : 0.f;
+        // 1 % covers the roundings of the bound itself
+        const float dev = 1.01f * (fmaf(er, fmaf(2.f, br, er), e2 * fmaf(2.f, bd, e2)) + 16.f * u * m);
+        if (n32 && n == last) {
+            if (!(m - dev > F.R2 * (1.f + 2.f * u))) return false;
+        } else if (!(m + dev < F.R2 * (1.f - 2.f * u))) {
+            return false;
+        }
+    }
+    return true;
+}
+
 // Re-render of one pixel by one warp (all 32 lanes call), with the oracle's
 // formulas for the sample positions (the reference sequence of steps) in FP64;
 // a march or bisection sample is classified in FP32 and again in FP64 only
@@ -485,7 +577,8 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
 }
 
 // Recheck entries of one warp are staged in shared memory.  At the end of its
-// tile the warp rechecks them itself in FP64 (recheck_staged): that FP64 work
+// tile the warp rechecks them itself (recheck_staged): those whose FP32 count a
+// rounding bound proves are done, the others are evaluated in FP64, which
 // overlaps with the FP32 march of the other warps on the SM instead of running
 // as a pass of its own after the march.  A tile that fills the stage
 // (kQStage entries per warp; a round adds at most 64) appends the staged
@@ -498,16 +591,17 @@ constexpr int kQStage = 256;
 constexpr float kFarT = 1e18f;
 
 // Append a warp's staged entries qs[0, qn) to the recheck queue (qn warp-uniform)
-// and count them as rechecks; entries beyond the queue's capacity re-render
+// and count those from `counted` on as rechecks; entries beyond the queue's capacity re-render
 // their pixel in FP64.
-__device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch &sc, const int4 *qs, int qn)
+__device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch &sc, const int4 *qs, int qn,
+                                             int counted)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
     unsigned base = 0;
     if (lane == 0) {
         base = atomicAdd(&sc.ctr->queue_count, (unsigned)qn);
-        atomicAdd(&sc.ctr->stats[4], (unsigned long long)qn);
+        atomicAdd(&sc.ctr->stats[4], (unsigned long long)(qn - counted));
     }
     base = __shfl_sync(kFull, base, 0);
     for (int i = lane; i < qn; i += 32) {
@@ -522,15 +616,57 @@ __device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch 
     __syncwarp();
 }
 
-// FP64 recheck of a warp's staged entries qs[0, qn) (qn warp-uniform), one per
-// lane, counted as rechecks.
-template <int SQ, int MOD>
-__device__ __forceinline__ void recheck_staged(const FrameDesc &fd, const Scratch &sc, const int4 *qs, int qn)
+// Recheck of a warp's staged entries qs[0, qn) (qn warp-uniform), counted as
+// rechecks from entry `counted` on: entries whose FP32 count is certain are done;
+// the others are gathered at the front and rechecked in FP64 in full batches of
+// 32 (an FP64 warp instruction takes the same time for one lane as for 32).
+// Returns how many are left in qs (fewer than 32); they stay staged for the
+// warp's next tile or go to the recheck queue (flush_rest).
+template <int SQ, int MOD, bool AXIS>
+__device__ __forceinline__ int recheck_staged(const FrameDesc &fd, const Scratch &sc, int4 *qs, int qn, int counted)
 {
     const int lane = threadIdx.x & 31;
     __syncwarp();
-    if (lane == 0) atomicAdd(&sc.ctr->stats[4], (unsigned long long)qn);
-    for (int i = lane; i < qn; i += 32) recheck_entry<SQ, MOD>(fd, sc, qs[i]);
+    if (lane == 0) atomicAdd(&sc.ctr->stats[4], (unsigned long long)(qn - counted));
+    int out = counted;
+    for (int base = counted; base < qn; base += 32) {
+        const int i = base + lane;
+        int4 e = make_int4(0, 0, 0, 0);
+        bool keep = false;
+        if (i < qn) {
+            e = qs[i];
+            keep = !count_certain<SQ, MOD, AXIS>(fd, e.z & 0xffff, e.z >> 16, e.y & 0xffff, e.w);
+        }
+        const unsigned m = __ballot_sync(kFull, keep);
+        if (keep) qs[out + __popc(m & ((1u << lane) - 1u))] = e;  // out <= base: read by now
+        out += __popc(m);
+        __syncwarp();
+        if (out >= 32) {  // fewer than 32 were left, at most 32 came: one batch
+            out -= 32;
+            recheck_entry<SQ, MOD>(fd, sc, qs[out + lane]);
+            __syncwarp();
+        }
+    }
+    return out;
+}
+
+// The entries a warp has left (already counted), to the recheck queue.
+__device__ __forceinline__ void flush_rest(const FrameDesc &fd, const Scratch &sc, const int4 *qs, int qn)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    unsigned base = 0;
+    if (lane == 0 && qn > 0) base = atomicAdd(&sc.ctr->queue_count, (unsigned)qn);
+    base = __shfl_sync(kFull, base, 0);
+    if (lane < qn) {
+        const int4 e = qs[lane];
+        if (base + (unsigned)lane < sc.queue_cap) {
+            sc.queue[base + lane] = e;
+        } else {
+            atomicAdd(&sc.ctr->stats[7], 1ull);
+            mark_dirty(fd, sc, e.x);
+        }
+    }
     __syncwarp();
 }
 
@@ -545,7 +681,8 @@ __device__ __forceinline__ void recheck_staged(const FrameDesc &fd, const Scratc
 // itself in sc.part_hit.
 template <int SQ, int MOD, bool RECHECK, bool AXIS = false, bool SPLIT = false>
 __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConsts &P, const Scratch &sc, unsigned tile,
-                                            LaneStats &st, int4 *qs = nullptr, int kb = 0, int ke = 0)
+                                            LaneStats &st, int4 *qs = nullptr, int *left = nullptr, int kb = 0,
+                                            int ke = 0)
 {
     const FrameT<float> &F = fd.f;
     const int lane = threadIdx.x & 31;
@@ -612,7 +749,7 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
     }
     const bool boxa = acta, boxb = actb;
     int suma = 0, sumb = 0, maxa = 0, maxb = 0, kfa = -1, kfb = -1;
-    int qn = 0;  // staged recheck entries (warp-uniform)
+    int qn = RECHECK ? *left : 0, counted = qn;  // staged recheck entries (warp-uniform); left: of earlier tiles
     const int k0 = SPLIT ? kb : 0, k1 = SPLIT ? ke : N + 1;
     float2 kf = make_float2((float)k0, (float)k0);
     // `more`: some ray of the warp still marches.  It changes only in a round
@@ -643,8 +780,8 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
             if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), xyb, inb ? 0 : cb + 1);
             qn += nq;
             if (qn > kQStage - 64) {
-                flush_staged(fd, sc, qs, qn);
-                qn = 0;
+                flush_staged(fd, sc, qs, qn, counted);
+                qn = counted = 0;
             }
         }
         // ina / inb imply acta / actb (they start equal and only clear)
@@ -664,7 +801,7 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
             more = __any_sync(kFull, acta || actb);
         }
     }
-    if (RECHECK && qn > 0) recheck_staged<SQ, MOD>(fd, sc, qs, qn);
+    if (RECHECK) *left = qn > counted ? recheck_staged<SQ, MOD, AXIS>(fd, sc, qs, qn, counted) : qn;
     const bool hita = kfa >= 0, hitb = kfb >= 0;
     // iterations = sum of (escape count) over escaped samples + max_iter per inside sample
     //            = sum of bounded steps + number of escaped samples
@@ -711,7 +848,8 @@ __device__ __forceinline__ void march2_tile(const FrameDesc &fd, const PairConst
 // the loop without it is the shorter one).  box: the warp's, in shared memory.
 template <int SQ, int MOD, bool RECHECK, bool AXIS, bool SPLIT, bool SETTLE>
 __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConsts &P, const Scratch &sc, unsigned tile,
-                                            LaneStats &st, TileBox &box, int4 *qs = nullptr, int kb = 0, int ke = 0)
+                                            LaneStats &st, TileBox &box, int4 *qs = nullptr, int *left = nullptr,
+                                            int kb = 0, int ke = 0)
 {
     const FrameT<float> &F = fd.f;
     const int lane = threadIdx.x & 31;
@@ -775,7 +913,7 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     }
     const bool boxa = acta, boxb = actb;
     int suma = 0, sumb = 0, maxa = 0, maxb = 0, kfa = -1, kfb = -1;
-    int qn = 0;  // staged recheck entries (warp-uniform)
+    int qn = RECHECK ? *left : 0, counted = qn;  // staged recheck entries (warp-uniform); left: of earlier tiles
     const int k0 = SPLIT ? kb : 0, k1 = SPLIT ? ke : N + 1;
     const float2 far = make_float2(kFarT, kFarT);
     bool more = __any_sync(kFull, acta || actb);
@@ -850,8 +988,8 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
                 if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), xyb, inb ? 0 : cb + 1);
                 qn += nqa + __popc(bb);
                 if (qn > kQStage - 64) {
-                    flush_staged(fd, sc, qs, qn);
-                    qn = 0;
+                    flush_staged(fd, sc, qs, qn, counted);
+                    qn = counted = 0;
                 }
             }
             {
@@ -864,8 +1002,8 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
                 if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k2 | (kMarchSample << 16), xyb, inb2 ? 0 : cb2 + 1);
                 qn += nqa + __popc(bb);
                 if (qn > kQStage - 64) {
-                    flush_staged(fd, sc, qs, qn);
-                    qn = 0;
+                    flush_staged(fd, sc, qs, qn, counted);
+                    qn = counted = 0;
                 }
             }
         }
@@ -899,7 +1037,7 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
             more = __any_sync(kFull, acta || actb);
         }
     }
-    if (RECHECK && qn > 0) recheck_staged<SQ, MOD>(fd, sc, qs, qn);
+    if (RECHECK) *left = qn > counted ? recheck_staged<SQ, MOD, AXIS>(fd, sc, qs, qn, counted) : qn;
     const bool hita = kfa >= 0, hitb = kfb >= 0;
     const int nesca = (hita ? kfa : k1) - k0, nescb = (hitb ? kfb : k1) - k0;
     if constexpr (SPLIT) {  // this range's partial result per ray (see march_merge_kernel)

@@ -181,6 +181,8 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 5 : 4)  // the general form kee
     march2_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
 {
     __shared__ int4 stage[RECHECK ? kBlock / 32 : 1][RECHECK ? kQStage : 1];  // recheck entries, per warp
+    int4 *qs = stage[RECHECK ? threadIdx.x >> 5 : 0];
+    int left = 0;  // entries staged by the warp's earlier tiles
     const int lane = threadIdx.x & 31;
     const unsigned ntiles = subset_tiles(fd, (unsigned)fd.tiles_x * (unsigned)fd.tiles_y);
     for (;;) {
@@ -191,9 +193,10 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 5 : 4)  // the general form kee
         tile = subset_tile(fd, tile);
         // counters are added per tile, so none stays live across the march loop
         LaneStats st;
-        march2_tile<SQ, MOD, RECHECK, AXIS>(fd, fd.p2, sc, tile, st, stage[RECHECK ? threadIdx.x >> 5 : 0]);
+        march2_tile<SQ, MOD, RECHECK, AXIS>(fd, fd.p2, sc, tile, st, qs, &left);
         flush_lane_stats<false>(sc, st, true);
     }
+    if (RECHECK) flush_rest(fd, sc, qs, left);
 }
 
 // march2_kernel with two samples of each ray per round (march4_tile).  Its
@@ -204,6 +207,8 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_kernel(const __gr
                                                                       const Scratch sc)
 {
     __shared__ int4 stage[RECHECK ? kBlock / 32 : 1][RECHECK ? kQStage : 1];  // recheck entries, per warp
+    int4 *qs = stage[RECHECK ? threadIdx.x >> 5 : 0];
+    int left = 0;  // entries staged by the warp's earlier tiles
     __shared__ TileBox box[kBlock / 32];
     const int lane = threadIdx.x & 31;
     const unsigned ntiles = subset_tiles(fd, (unsigned)fd.tiles_x * (unsigned)fd.tiles_y);
@@ -214,10 +219,10 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_kernel(const __gr
         if (tile >= ntiles) break;
         tile = subset_tile(fd, tile);
         LaneStats st;
-        march4_tile<SQ, MOD, RECHECK, AXIS, false, SETTLE>(fd, fd.p2, sc, tile, st, box[threadIdx.x >> 5],
-                                            stage[RECHECK ? threadIdx.x >> 5 : 0]);
+        march4_tile<SQ, MOD, RECHECK, AXIS, false, SETTLE>(fd, fd.p2, sc, tile, st, box[threadIdx.x >> 5], qs, &left);
         flush_lane_stats<false>(sc, st, true);
     }
+    if (RECHECK) flush_rest(fd, sc, qs, left);
 }
 
 // ---------------------------------------------------------------------------
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 5 : 4) march2_split_kernel(cons
         const unsigned r = item / ntiles, tile = subset_tile(fd, item % ntiles);
         const int kb = (int)r * fd.k_chunk, ke = min(kb + fd.k_chunk, fd.N + 1);
         LaneStats st;
-        march2_tile<SQ, MOD, false, AXIS, true>(fd, fd.p2, sc, tile, st, nullptr, kb, ke);
+        march2_tile<SQ, MOD, false, AXIS, true>(fd, fd.p2, sc, tile, st, nullptr, nullptr, kb, ke);
     }
 }
 
@@ -265,7 +270,7 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_split_kernel(cons
         const unsigned r = item / ntiles, tile = subset_tile(fd, item % ntiles);
         const int kb = (int)r * fd.k_chunk, ke = min(kb + fd.k_chunk, fd.N + 1);
         LaneStats st;
-        march4_tile<SQ, MOD, false, AXIS, true, false>(fd, fd.p2, sc, tile, st, box[threadIdx.x >> 5], nullptr, kb, ke);
+        march4_tile<SQ, MOD, false, AXIS, true, false>(fd, fd.p2, sc, tile, st, box[threadIdx.x >> 5], nullptr, nullptr, kb, ke);
     }
 }
 

@@ -153,7 +153,9 @@ __device__ __noinline__ void march_item4(const FrameDesc &fd, const Scratch &sc,
                                          int4 *stage)
 {
     LaneStats st;
-    march4_tile<0, 0, RECHECK, AXIS, false, true>(fd, fd.p2, sc, tile, st, box, stage);
+    int left = 0;
+    march4_tile<0, 0, RECHECK, AXIS, false, true>(fd, fd.p2, sc, tile, st, box, stage, &left);
+    if (RECHECK) flush_rest(fd, sc, stage, left);
     flush_lane_stats<false>(sc, st, true);
 }
 
@@ -161,7 +163,9 @@ template <bool RECHECK, bool AXIS>
 __device__ __noinline__ void march_item2(const FrameDesc &fd, const Scratch &sc, unsigned tile, int4 *stage)
 {
     LaneStats st;
-    march2_tile<0, 0, RECHECK, AXIS>(fd, fd.p2, sc, tile, st, stage);
+    int left = 0;
+    march2_tile<0, 0, RECHECK, AXIS>(fd, fd.p2, sc, tile, st, stage, &left);
+    if (RECHECK) flush_rest(fd, sc, stage, left);
     flush_lane_stats<false>(sc, st, true);
 }
 
