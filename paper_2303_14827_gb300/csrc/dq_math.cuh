@@ -236,22 +236,6 @@ __device__ __forceinline__ int classify_scalar_axis(T (&z)[8], const FrameT<T> &
     return 0;
 }
 
-// classify_scalar that also reports whether any tested modulus, up to and
-// including the escaping one, lay within F.margin of R^2.
-template <typename T, int SQ, int MOD>
-__device__ __forceinline__ int classify_scalar_margin(T (&z)[8], const FrameT<T> &F, int max_iter, bool &marginal)
-{
-    T sp = dq_sp<T>(z);
-    marginal = false;
-    const bool long_orbits = max_iter > late_step<MOD>();  // steps past late_step count as marginal
-    for (int n = 1; n <= max_iter; ++n) {
-        const T m = dq_iter<T, SQ, MOD>(z, z, sp, F.c);
-        marginal = marginal || fabs(m - F.R2) <= F.margin || (long_orbits && n > late_step<MOD>());
-        if (m > F.R2) return n;
-    }
-    return 0;
-}
-
 template <typename T, int SQ, int MOD>
 __device__ __forceinline__ int classify_scalar(T (&z)[8], const FrameT<T> &F, int max_iter)
 {

@@ -285,15 +285,13 @@ __device__ __forceinline__ void ray_clip64(const FrameDesc &fd, const double (&w
     }
 }
 
-// FP64 recheck of one queued sample {pixel, k | b << 16, path, n32}: the sample
-// is placed on its FP64 ray (a march sample k, with x | y << 16 in place of the
-// path, or bisection level b of the bracket (k - 1, k) replayed from the path
-// bits), classified in FP64, and the pixel is queued for an FP64 re-render when
-// its FP64 escape count differs from the FP32 one.  Positions may differ from
-// the reference formula's in the last place, as the FP64 iteration's contracted
-// FMAs already do.
-template <int SQ, int MOD>
-__device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch &sc, int4 e)
+// FP64 slice point of one queued sample {pixel, k | b << 16, path, n32} on its
+// FP64 ray: a march sample k (with x | y << 16 in place of the path), or
+// bisection level b of the bracket (k - 1, k) replayed from the path bits.
+// Positions may differ from the reference formula's in the last place, as the
+// FP64 iteration's contracted FMAs already do.  Components 3..7 of an
+// axis-aligned slice are set to zero.
+__device__ __forceinline__ void entry_point64(const FrameDesc &fd, int4 e, double (&z)[8])
 {
     const FrameT<double> &F = fd.d;
     const int pixel = e.x, k = e.y & 0xffff, b = e.y >> 16;
@@ -317,46 +315,118 @@ __device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch
         }
         t = lo + 0.5 * (hi - lo);
     }
-    double z[8];
-    int n64;
-    if (fd.axis_slice) {
-        // components 3..7 of the slice point are zero, so the first step takes
-        // the axis form, whose operations are those of dq_iter on those zeros
+    auto comp = [&](int j) {
+        z[j] = fma(t, fma(w[0], F.E[0][j], fma(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
+    };
 #pragma unroll
-        for (int j = 0; j < 3; ++j)
-            z[j] = fma(t, fma(w[0], F.E[0][j], fma(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
+    for (int j = 0; j < 3; ++j) comp(j);
 #pragma unroll
-        for (int j = 3; j < 8; ++j) z[j] = 0.0;
-        n64 = classify_scalar_axis<double, SQ, MOD>(z, F, fd.max_iter);
-    } else {
+    for (int j = 3; j < 8; ++j) z[j] = 0.0;
+    if (!fd.axis_slice) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            z[j] = fma(t, fma(w[0], F.E[0][j], fma(w[1], F.E[1][j], w[2] * F.E[2][j])), F.A[j]);
-        n64 = classify_scalar<double, SQ, MOD>(z, F, fd.max_iter);
+        for (int j = 3; j < 8; ++j) comp(j);
     }
-    if (n64 != e.w) mark_dirty(fd, sc, pixel);
 }
 
-// Is the FP32 escape count n32 of march sample k of pixel (x, y) certain?  The
-// sample's FP32 orbit is run again beside a bound of its distance from the exact
-// orbit, (er, ed) on the real and dual halves: the rounding of the sample's
-// position, then per step
+// Escape count of a FP64 slice point, in FP64.  An axis-aligned slice takes the
+// axis form of the first step, whose operations are those of dq_iter on the
+// zero components: the same iterate.
+template <int SQ, int MOD>
+__device__ __forceinline__ int count64(const FrameDesc &fd, double (&z)[8])
+{
+    return fd.axis_slice ? classify_scalar_axis<double, SQ, MOD>(z, fd.d, fd.max_iter)
+                         : classify_scalar<double, SQ, MOD>(z, fd.d, fd.max_iter);
+}
+
+// FP64 recheck of one queued sample: the pixel is queued for an FP64 re-render
+// when the sample's FP64 escape count differs from its FP32 one.
+template <int SQ, int MOD>
+__device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch &sc, int4 e)
+{
+    double z[8];
+    entry_point64(fd, e, z);
+    if (count64<SQ, MOD>(fd, z) != e.w) mark_dirty(fd, sc, e.x);
+}
+
+// Escape count of a sample by its FP32 orbit beside a bound (er, ed) of that
+// orbit's distance from the exact one on the real and dual halves: the given
+// rounding of the starting point z, then per step
 //     er <- 2 |z_r| er + er^2 + rounding,  ed <- 2 (|z_r| ed + |z_d| er + er ed) + rounding
 // (algebraic square; quaternion norms multiply), so a step's exact modulus lies
 // within 2 (|z_r| er + |z_d| ed) + er^2 + ed^2 of the FP32 one.  Where every
-// step up to n32 decides clear of that, FP64 can only give n32 too, and the
-// sample needs no FP64 evaluation.  A sample is flagged within 1e-3 of R^2
-// (by default); after the one to three steps of most flagged samples the bound
-// is 1e-5 to 1e-4 of it.
+// step decides clear of that, the count is the exact sample's and FP64 can only
+// give the same: `certain`.  Otherwise the count returned means nothing.
 //
-// Rounding, with u = 2^-24: the camera map's constants and three FMAs put w
-// within 8 u m of the exact direction, m = |fwd| + |sx| + |sy| a bound of its
+// Rounding of a step, u = 2^-24, term by term of dq_iter: the real half errs by
+// at most u (5.1 |z_r|^2 + 4.3 |c|), the dual half by u (4.5 (|z_r|^2 + |z_d|^2)
+// + 4 |c|) (the rounding of c included); the modulus by 8 u of itself.
+template <int SQ, int MOD>
+__device__ __forceinline__ int count_bound(const FrameDesc &fd, float (&z)[8], float er, float ed, bool &certain)
+{
+    const FrameT<float> &F = fd.f;
+    constexpr float u = 5.9604645e-8f;
+    const float hi = F.R2 * (1.f + 2.f * u), lo = F.R2 * (1.f - 2.f * u);
+    float sp = dq_sp<float>(z);
+    float r2 = fmaf(z[0], z[0], sp), d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
+    float ar = sqrt_approx(r2), ad = sqrt_approx(d2);
+    certain = true;
+    for (int n = 1; n <= fd.max_iter; ++n) {
+        const float round = 5.6f * u * (r2 + d2 + fd.settle_cn);
+        const float ner = fmaf(er, fmaf(2.f, ar, er), round);
+        if (SQ == 0)
+            ed = fmaf(2.f, fmaf(ar, ed, fmaf(ad, er, er * ed)), round);
+        else
+            ed = fmaf(ed, fmaf(2.f, ad, ed), round);
+        er = ner;
+        dq_iter<float, SQ, MOD>(z, z, sp, F.c);
+        r2 = fmaf(z[0], z[0], sp);
+        d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
+        ar = sqrt_approx(r2);
+        ad = sqrt_approx(d2);
+        const float m = MOD == 0 ? r2 + d2 : r2;
+        // 1 % covers the roundings of the bound itself
+        float dev = er * fmaf(2.f, ar, er);
+        if (MOD == 0) dev = fmaf(ed, fmaf(2.f, ad, ed), dev);
+        dev = fmaf(1.01f, dev, 10.f * u * m);
+        if (m - dev > hi) return n;
+        if (!(m + dev < lo)) {
+            certain = false;
+            return 0;
+        }
+    }
+    return 0;
+}
+
+// count_bound of a FP64 point: its FP32 image lies within u of every component.
+template <int SQ, int MOD>
+__device__ __forceinline__ int count_bound64(const FrameDesc &fd, const double (&z64)[8], bool &certain)
+{
+    float z[8];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) z[j] = (float)z64[j];
+#pragma unroll
+    for (int j = 3; j < 8; ++j) z[j] = 0.f;
+    if (!fd.axis_slice) {
+#pragma unroll
+        for (int j = 3; j < 8; ++j) z[j] = (float)z64[j];
+    }
+    float n2 = z[0] * z[0];
+#pragma unroll
+    for (int j = 1; j < 8; ++j) n2 = fmaf(z[j], z[j], n2);
+    const float e0 = 6.1e-8f * sqrt_approx(n2);
+    return count_bound<SQ, MOD>(fd, z, e0, e0, certain);
+}
+
+// Is the FP32 escape count n32 of march sample k of pixel (x, y) certain?  The
+// sample is placed by FP32 arithmetic with a bound of its rounding: with
+// u = 2^-24, the camera map's constants and three FMAs put w within 8 u m of
+// the exact direction, m = 1 + |sx| + |sy| + 2 (|sxb| + |syb|) a bound of its
 // terms; a face parameter tau = (face - eye) / w then lies within
 // |tau| (8 u m / |w_a| + 8 u) + 3 u (|face| + |eye|) / |w_a| of its exact
-// value, and the entry (a maximum) and
-// exit (a minimum) within what the faces' upper and lower values give; the
-// position A + tau W adds 4 u of its terms.  A step's FMAs, each rounding at
-// most u of a term bounded by |z|^2 + |c|, err by less than 16 u of that.
+// value, and the entry (a maximum) and exit (a minimum) within what the faces'
+// upper and lower values give; the position A + tau W adds 8 u of its terms.
+// A sample is flagged within 1e-3 of R^2 (by default); after the one to three
+// steps of most flagged samples the bound is 1e-5 to 1e-4 of it.
 template <int SQ, int MOD, bool AXIS>
 __device__ __forceinline__ bool count_certain(const FrameDesc &fd, int x, int y, int k, int n32)
 {
@@ -401,38 +471,15 @@ __device__ __forceinline__ bool count_certain(const FrameDesc &fd, int x, int y,
             for (int j = 3; j < 8; ++j) z[j] = 0.f;
         }
     }
-    float sp = dq_sp<float>(z), m = 0.f;
-    float r2 = fmaf(z[0], z[0], sp), d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
-    const int last = n32 ? n32 : fd.max_iter;
-    for (int n = 1; n <= last; ++n) {
-        const float ar = sqrt_approx(r2), ad = sqrt_approx(d2);
-        const float round = 16.f * u * (r2 + d2 + fd.settle_cn);
-        const float ner = fmaf(er, fmaf(2.f, ar, er), round);
-        if (SQ == 0)
-            ed = fmaf(2.f, fmaf(ar, ed, fmaf(ad, er, er * ed)), round);
-        else
-            ed = fmaf(ed, fmaf(2.f, ad, ed), round);
-        er = ner;
-        dq_iter<float, SQ, MOD>(z, z, sp, F.c);
-        r2 = fmaf(z[0], z[0], sp);
-        d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
-        m = MOD == 0 ? r2 + d2 : r2;
-        const float br = sqrt_approx(r2), bd = MOD == 0 ? sqrt_approx(d2) : 0.f, e2 = MOD == 0 ? ed : 0.f;
-        // 1 % covers the roundings of the bound itself
-        const float dev = 1.01f * (fmaf(er, fmaf(2.f, br, er), e2 * fmaf(2.f, bd, e2)) + 16.f * u * m);
-        if (n32 && n == last) {
-            if (!(m - dev > F.R2 * (1.f + 2.f * u))) return false;
-        } else if (!(m + dev < F.R2 * (1.f - 2.f * u))) {
-            return false;
-        }
-    }
-    return true;
+    bool certain;
+    const int n = count_bound<SQ, MOD>(fd, z, er, ed, certain);
+    return certain && n == n32;
 }
 
 // Re-render of one pixel by one warp (all 32 lanes call), with the oracle's
 // formulas for the sample positions (the reference sequence of steps) in FP64;
-// a march or bisection sample is classified in FP32 and again in FP64 only
-// when it is marginal (the premise of the recheck mode); the bisection runs
+// a march or bisection sample is classified in FP32 where the rounding bound
+// decides (count_bound), else in FP64; the bisection runs
 // five levels per round across the lanes; the normal is FP64.  The lanes classify 32 consecutive march samples at a time; a ballot
 // finds the first inside one and warp reductions give the largest escape count
 // before it, so the result and the iteration count are those of the
@@ -440,7 +487,7 @@ __device__ __forceinline__ bool count_certain(const FrameDesc &fd, int x, int y,
 // evaluations run on lanes 0..5.  Adds the iterations to its (per lane) and the
 // pixel to npx (lane 0).
 template <int SQ, int MOD>
-__device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, unsigned long long &its,
+__device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, TileBox &box, unsigned long long &its,
                                             unsigned long long &npx)
 {
     const FrameT<double> &F = fd.d;
@@ -455,35 +502,46 @@ __device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, unsi
         }
         const double delta = (t_out - t_in) / (double)fd.N;
         auto slice = [&](double t, double (&z)[8]) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
+            auto comp = [&](int j) {
                 z[j] = F.O[j] + (F.eye[0] + t * d[0]) * F.E[0][j] + (F.eye[1] + t * d[1]) * F.E[1][j] +
                        (F.eye[2] + t * d[2]) * F.E[2][j];
+            };
+#pragma unroll
+            for (int j = 0; j < 3; ++j) comp(j);
+#pragma unroll
+            for (int j = 3; j < 8; ++j) z[j] = 0.0;
+            if (!fd.axis_slice) {  // (zero on an axis-aligned slice)
+#pragma unroll
+                for (int j = 3; j < 8; ++j) comp(j);
+            }
         };
-        // FP64 classification; an axis-aligned slice takes the axis form of the
-        // first step (the same iterate, see classify_scalar_axis)
-        auto cls64 = [&](double (&z)[8]) {
-            return fd.axis_slice ? classify_scalar_axis<double, SQ, MOD>(z, F, fd.max_iter)
-                                 : classify_scalar<double, SQ, MOD>(z, F, fd.max_iter);
-        };
-        // a march sample: FP32 first, FP64 only when some FP32 modulus came within
-        // the recheck margin of R^2 (the premise of the recheck mode: outside the
-        // margin FP32 decides as FP64 does)
+        const float df[3] = {(float)d[0], (float)d[1], (float)d[2]};
+        tile_box(fd, true, df, (float)t_in, (float)t_out, false, df, 0.f, 0.f, box);
+        // a sample: by the FP32 orbit where its bound decides, else in FP64
         auto cls_march = [&](double t) {
             double z[8];
             slice(t, z);
-            float zf[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) zf[j] = (float)z[j];
-            bool marginal;
-            const int n32 = classify_scalar_margin<float, SQ, MOD>(zf, fd.f, fd.max_iter, marginal);
-            return marginal ? cls64(z) : n32;
+            bool certain;
+            const int n32 = count_bound64<SQ, MOD>(fd, z, certain);
+            return certain ? n32 : count64<SQ, MOD>(fd, z);
         };
         int esc_max = 0, n_prev = 0, k_first = -1;
+        unsigned w = 0;
         for (int k0 = 0; k0 <= fd.N; k0 += 32) {
             const int k = k0 + lane;
             const bool part = k <= fd.N;
-            const int n = part ? cls_march(t_in + (double)k * delta) : 1;
+            // the ray's settled samples (blocks of 16, chunks of 512: see
+            // settle.cuh) have their counts; the others are classified
+            if (k0 % kSettleChunk == 0) {
+                const int ke = min(k0 + kSettleChunk, fd.N + 1);
+                w = fd.axis_slice ? settle_chunk<SQ, MOD, true>(fd, box, k0, ke, kSettlePairs)
+                                  : settle_chunk<SQ, MOD, false>(fd, box, k0, ke, kSettlePairs);
+            }
+            const unsigned word = __shfl_sync(kFull, w, (k % kSettleChunk) / (2 * kSettlePairs));
+            int n = (int)((word >> (4 * ((k % (2 * kSettlePairs)) >> 1))) & 15u);
+            if (!part) n = 1;
+            if (n == 0) n = cls_march(t_in + (double)k * delta);
+            __syncwarp();
             const unsigned inside = __ballot_sync(kFull, part && n == 0);
             const int first = inside ? __ffs(inside) - 1 : 32;  // samples before it escaped
             if (part && lane <= first) its += n ? (unsigned)n : (unsigned)fd.max_iter;
@@ -648,6 +706,37 @@ __device__ __forceinline__ int recheck_staged(const FrameDesc &fd, const Scratch
         }
     }
     return out;
+}
+
+// Recheck of queue entries [base, base + 32) clipped to nq by one warp (all 32
+// lanes call), positions in FP64: entries whose FP32 count the rounding bound
+// proves are done, the others join those in qs[0, left) and are evaluated in
+// FP64 in full batches.  Returns the new number left in qs (room for 64).
+template <int SQ, int MOD>
+__device__ __forceinline__ int recheck_batch(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nq,
+                                             int4 *qs, int left)
+{
+    const int lane = threadIdx.x & 31;
+    int4 e = make_int4(0, 0, 0, 0);
+    bool keep = false;
+    if (base + lane < nq) {
+        e = __ldcg(sc.queue + base + lane);
+        double z[8];
+        entry_point64(fd, e, z);
+        bool certain;
+        const int n = count_bound64<SQ, MOD>(fd, z, certain);
+        keep = !(certain && n == e.w);
+    }
+    const unsigned m = __ballot_sync(kFull, keep);
+    if (keep) qs[left + __popc(m & ((1u << lane) - 1u))] = e;
+    left += __popc(m);
+    __syncwarp();
+    if (left >= 32) {
+        left -= 32;
+        recheck_entry<SQ, MOD>(fd, sc, qs[left + lane]);
+        __syncwarp();
+    }
+    return left;
 }
 
 // The entries a warp has left (already counted), to the recheck queue.

@@ -187,16 +187,17 @@ __device__ __noinline__ void bisect_item(const FrameDesc &fd, const Scratch &sc,
     flush_lane_stats<RECHECK>(sc, st, false);
 }
 
-__device__ __noinline__ void recheck_item(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nq)
+__device__ __noinline__ void recheck_item(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nq, int4 *stage)
 {
-    const int lane = threadIdx.x & 31;
-    if (base + lane < nq) recheck_entry<0, 0>(fd, sc, __ldcg(sc.queue + base + lane));
+    const int left = recheck_batch<0, 0>(fd, sc, base, nq, stage, 0);
+    if ((int)(threadIdx.x & 31) < left) recheck_entry<0, 0>(fd, sc, stage[threadIdx.x & 31]);
+    __syncwarp();
 }
 
-__device__ __noinline__ void fixup_item(const FrameDesc &fd, const Scratch &sc, unsigned i)
+__device__ __noinline__ void fixup_item(const FrameDesc &fd, const Scratch &sc, unsigned i, TileBox &box)
 {
     unsigned long long its = 0, npx = 0;
-    fixup_pixel<0, 0>(fd, __ldcg(sc.dirty_list + i), its, npx);
+    fixup_pixel<0, 0>(fd, __ldcg(sc.dirty_list + i), box, its, npx);
     flush_stat(&sc.ctr->stats[6], its);
     flush_stat(&sc.ctr->stats[5], npx);
 }
@@ -320,12 +321,12 @@ __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
             total = nh;
         } else if (ph == kPhaseRecheck) {
             const unsigned nq = ld_vol32(&b->q_total);
-            recheck_item(fd, sc, item, nq);
+            recheck_item(fd, sc, item, nq, s_stage[wib]);
             done_ctr = &b->q_done;
             n_items = min(32u, nq - item);
             total = nq;
         } else {
-            fixup_item(fd, sc, item);
+            fixup_item(fd, sc, item, s_box[wib]);
             done_ctr = &b->f_done;
             n_items = 1;
             total = ld_vol32(&b->f_total);
