@@ -417,6 +417,30 @@ __device__ __forceinline__ int count_bound64(const FrameDesc &fd, const double (
     return count_bound<SQ, MOD>(fd, z, e0, e0, certain);
 }
 
+// Lockstep classification of one sample per lane (classify_lockstep), FP64 by
+// the bound first: a lane whose count the FP32 orbit's bound proves needs no
+// FP64 iteration, and a warp iterates in FP64 only when some lane does.  FP32
+// samples are classified as they are.
+template <typename T, int SQ, int MOD, bool RECHECK>
+__device__ __forceinline__ int classify_sample(const FrameDesc &fd, T (&z)[8], bool part, bool &marginal)
+{
+    if constexpr (sizeof(T) == 8) {
+        static_assert(!RECHECK, "the recheck mode classifies in FP32");
+        marginal = false;
+        bool certain = true;
+        int n = 1;
+        if (part) n = count_bound64<SQ, MOD>(fd, z, certain);
+        const bool again = part && !certain;
+        if (__any_sync(kFull, again)) {
+            const int m = classify_lockstep<T, SQ, MOD, false>(z, fd.d, fd.max_iter, again, marginal);
+            if (again) n = m;
+        }
+        return n;
+    } else {
+        return classify_lockstep<T, SQ, MOD, RECHECK>(z, frame<T>(fd), fd.max_iter, part, marginal);
+    }
+}
+
 // Is the FP32 escape count n32 of march sample k of pixel (x, y) certain?  The
 // sample is placed by FP32 arithmetic with a bound of its rounding: with
 // u = 2^-24, the camera map's constants and three FMAs put w within 8 u m of
@@ -1194,6 +1218,58 @@ __device__ __forceinline__ void normal_shade(const FrameDesc &fd, const FrameT<T
     }
 }
 
+// FP64 normals and shading of the hits of the lanes in `mask` (pixel (x, y),
+// depth and n* on those lanes; all 32 lanes call): five hits at a time, the six
+// field evaluations of a hit on six lanes, on the hit's FP64 ray.  The normals
+// of a recheck frame with more than late_step steps come here.  An FP64 warp
+// instruction takes the same time for one lane as for 32, so evaluating the six
+// in turn on the hits' own lanes, or on the four lanes of a hit's group, wasted
+// the lanes of the other hits (512 x 512, max_iter 24, 55 % of the hits late:
+// bisection pass 0.74 -> 0.63 ms).
+template <int SQ, int MOD>
+__device__ __forceinline__ void late_normals(const FrameDesc &fd, unsigned mask, int x, int y, double depth, int n_star,
+                                             LaneStats &st)
+{
+    const FrameT<double> &F = fd.d;
+    const int lane = threadIdx.x & 31;
+    const int grp = lane / 6, q = lane - 6 * grp;  // lanes 30 and 31 idle
+    while (mask) {
+        int src = -1, nmax = 0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const int b = mask ? __ffs(mask) - 1 : -1;
+            mask &= mask - 1;
+            if (grp == j) src = b;
+            if (b >= 0) nmax = max(nmax, __shfl_sync(kFull, n_star, b));
+        }
+        const int from = src < 0 ? 0 : src;
+        const int hx = __shfl_sync(kFull, x, from), hy = __shfl_sync(kFull, y, from);
+        const int ns = __shfl_sync(kFull, n_star, from);
+        const double t = __shfl_sync(kFull, depth, from);
+        double d[3], D[8], t_in, t_out;
+        camera_clip<double>(F, fd.W, fd.H, hx, hy, d, t_in, t_out);
+        slice_dir<double>(F, d, D);
+        const int a = q >> 1;
+        const double hs = (q & 1) == 0 ? F.h : -F.h;
+        double z[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z[i] = fma(hs, F.E[a][i], fma(t, D[i], F.A[i]));
+        double sp = dq_sp<double>(z);
+        for (int n = 0; n < nmax; ++n)
+            if (n < ns) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
+        const double fv = modulus<double, MOD>(z);
+        const unsigned bad = __ballot_sync(kFull, !(fv <= normal_fmax(0.0)));
+        double f[6];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) f[i] = __shfl_sync(kFull, fv, min(6 * grp, 24) + i);
+        if (src >= 0 && q == 0) {
+            const double g[3] = {f[0] - f[1], f[2] - f[3], f[4] - f[5]};
+            st.niters += 6ull * (unsigned)ns;
+            shade_write<double>(fd, F, hx, hy, ns, t, g, ((bad >> (6 * grp)) & 63u) != 0, d);
+        }
+    }
+}
+
 // Bisection, normal and shading of hit-list entries [base, base + 32) clipped to
 // nhits, one per lane (see bisect_kernel); all 32 lanes call.
 template <typename T, int SQ, int MOD, bool RECHECK>
@@ -1239,7 +1315,7 @@ __device__ __forceinline__ void bisect_chunk(const FrameDesc &fd, const Scratch 
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) z[i] = dfma(lo, D[i], F.A[i]);
-            n = classify_lockstep<T, SQ, MOD, false>(z, F, fd.max_iter, bis, mg);
+            n = classify_sample<T, SQ, MOD, false>(fd, z, bis, mg);
         }
         if (bis) n_lo = n;
     }
@@ -1251,7 +1327,7 @@ __device__ __forceinline__ void bisect_chunk(const FrameDesc &fd, const Scratch 
 #pragma unroll
         for (int i = 0; i < 8; ++i) z[i] = dfma(mid, D[i], F.A[i]);
         bool mg;
-        const int n = classify_lockstep<T, SQ, MOD, RECHECK>(z, F, fd.max_iter, bis, mg);
+        const int n = classify_sample<T, SQ, MOD, RECHECK>(fd, z, bis, mg);
         if (RECHECK) {
             const bool push = bis && mg;
             if (warp_push(push, make_int4(pixel, k_first | (b << 16), (int)path, n), sc.queue, sc.queue_cap,
@@ -1279,13 +1355,8 @@ __device__ __forceinline__ void bisect_chunk(const FrameDesc &fd, const Scratch 
     // FP64 (on the FP64 ray, at the bisection's depth); the others in FP32
     const bool n64 = RECHECK && sizeof(T) == 4 && part && n_lo > late_step<MOD>();
     normal_shade<T, SQ, MOD>(fd, F, x, y, d, D, depth, n_lo, part && !n64, st);
-    if (RECHECK && sizeof(T) == 4 && __any_sync(kFull, n64)) {
-        const FrameT<double> &Fd = fd.d;
-        double dd[3] = {0.0, 0.0, 1.0}, ti = 0.0, to = 0.0, Dd[8];
-        if (n64) camera_clip<double>(Fd, fd.W, fd.H, x, y, dd, ti, to);
-        slice_dir<double>(Fd, dd, Dd);
-        normal_shade<double, SQ, MOD>(fd, Fd, x, y, dd, Dd, (double)depth, n_lo, n64, st);
-    }
+    if constexpr (RECHECK && sizeof(T) == 4)
+        late_normals<SQ, MOD>(fd, __ballot_sync(kFull, n64), x, y, (double)depth, n_lo, st);
     st.iters += iters;
     st.samples += samples;
 }
@@ -1406,7 +1477,7 @@ __device__ __forceinline__ void bisect_group(const FrameDesc &fd, const Scratch 
 #pragma unroll
         for (int i = 0; i < 8; ++i) z[i] = dfma(pos, D[i], F.A[i]);
         bool mg;
-        const int n = classify_lockstep<T, SQ, MOD, RECHECK>(z, F, fd.max_iter, act, mg);
+        const int n = classify_sample<T, SQ, MOD, RECHECK>(fd, z, act, mg);
         if (b0 == 0 && lo_in_round0) {
             const int nl = __shfl_sync(kFull, n, gb + L - 1);
             if (bis) n_lo = nl;
@@ -1447,13 +1518,8 @@ __device__ __forceinline__ void bisect_group(const FrameDesc &fd, const Scratch 
     // bisect_chunk), the others in T
     const bool n64 = RECHECK && sizeof(T) == 4 && part && n_lo > late_step<MOD>();
     group_normal<T, SQ, MOD, L>(fd, F, x, y, d, D, depth, n_lo, part && !n64, st);
-    if (RECHECK && sizeof(T) == 4 && __any_sync(kFull, n64)) {
-        const FrameT<double> &Fd = fd.d;
-        double dd[3] = {0.0, 0.0, 1.0}, ti = 0.0, to = 0.0, Dd[8];
-        if (n64) camera_clip<double>(Fd, fd.W, fd.H, x, y, dd, ti, to);
-        slice_dir<double>(Fd, dd, Dd);
-        group_normal<double, SQ, MOD, L>(fd, Fd, x, y, dd, Dd, (double)depth, n_lo, n64, st);
-    }
+    if constexpr (RECHECK && sizeof(T) == 4)
+        late_normals<SQ, MOD>(fd, __ballot_sync(kFull, n64 && j == 0), x, y, (double)depth, n_lo, st);
     if (part && j == 0) {
         st.iters += iters;
         st.samples += samples;

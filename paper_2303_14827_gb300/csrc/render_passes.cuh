@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kBlock) march_kernel(const __grid_constant__ F
                 const T t = dfma(T(k), delta, t_in);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) z[i] = dfma(t, D[i], F.A[i]);
-                n = classify_lockstep<T, SQ, MOD, RECHECK>(z, F, fd.max_iter, active, mg);
+                n = classify_sample<T, SQ, MOD, RECHECK>(fd, z, active, mg);
             }
             if (RECHECK) {
                 const bool push = active && mg;
