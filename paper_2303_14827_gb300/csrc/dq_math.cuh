@@ -132,6 +132,7 @@ __device__ __forceinline__ int classify_lockstep(T (&z)[8], const FrameT<T> &F, 
     T sp = dq_sp<T>(z);
     T w[8];
     // two steps per trip, z -> w -> z, with the escape test after each
+#pragma unroll 1
     for (int n = 0; n < max_iter; n += 2) {
         T m = dq_iter<T, SQ, MOD>(z, w, sp, F.c);
         if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
@@ -178,6 +179,7 @@ __device__ __forceinline__ int classify_lockstep_it1(T (&z)[8], const FrameT<T> 
     int cnt = alive ? 1 : 0;
     T w[8];
     if (__any_sync(0xffffffffu, alive)) {
+#pragma unroll 1
         for (int n = 1; n < max_iter; n += 2) {
             m = dq_iter<T, SQ, MOD>(z, w, sp, F.c);
             if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
@@ -231,6 +233,7 @@ __device__ __forceinline__ int classify_scalar_axis(T (&z)[8], const FrameT<T> &
     T sp = dfma(z[2], z[2], z[1] * z[1]);
     if (max_iter < 1) return 0;
     if (dq_iter_axis_first<T, MOD>(z, z, sp, F.c) > F.R2) return 1;
+#pragma unroll 1
     for (int n = 2; n <= max_iter; ++n)
         if (dq_iter<T, SQ, MOD>(z, z, sp, F.c) > F.R2) return n;
     return 0;
@@ -240,6 +243,7 @@ template <typename T, int SQ, int MOD>
 __device__ __forceinline__ int classify_scalar(T (&z)[8], const FrameT<T> &F, int max_iter)
 {
     T sp = dq_sp<T>(z);
+#pragma unroll 1
     for (int n = 1; n <= max_iter; ++n)
         if (dq_iter<T, SQ, MOD>(z, z, sp, F.c) > F.R2) return n;
     return 0;
@@ -498,6 +502,7 @@ __device__ __forceinline__ void classify_lockstep2(float2 (&z)[8], const PairCon
         }
     }
     // two steps per trip, z -> w -> z, with the escape test after each
+#pragma unroll 1
     for (int n = n0; n < max_iter; n += 2) {
         test(dq_iter2<SQ, MOD>(z, w, sp, P));
         v = __any_sync(0xffffffffu, aa || ab);
@@ -552,6 +557,7 @@ __device__ __forceinline__ void classify_lockstep2_it1(float2 (&z)[8], const Pai
     bool v = __any_sync(0xffffffffu, aa || ab);
     if (v) {
         // two steps per trip, z -> w -> z, with the escape test after each
+#pragma unroll 1
         for (int n = 1; n < max_iter; n += 2) {
             test(dq_iter2<SQ, MOD>(z, w, sp, P));
             v = __any_sync(0xffffffffu, aa || ab);
@@ -629,6 +635,7 @@ __device__ __forceinline__ void classify_lockstep4_axis(float2 (&z)[8], float2 (
             if (v) n0 = 2;
         }
     }
+#pragma unroll 1
     for (int n = n0; n < max_iter; n += 2) {
         test(dq_iter2<SQ, MOD>(z, w, sp, P), dq_iter2<SQ, MOD>(y, u, sq, P));
         v = __any_sync(0xffffffffu, aa || ab || aa2 || ab2);
@@ -694,6 +701,7 @@ __device__ __forceinline__ void classify_lockstep4_it1(float2 (&z)[8], float2 (&
     }
     bool v = __any_sync(0xffffffffu, aa || ab || aa2 || ab2);
     if (v) {
+#pragma unroll 1
         for (int n = 1; n < max_iter; n += 2) {
             test(dq_iter2<SQ, MOD>(z, w, sp, P), dq_iter2<SQ, MOD>(y, u, sq, P));
             v = __any_sync(0xffffffffu, aa || ab || aa2 || ab2);

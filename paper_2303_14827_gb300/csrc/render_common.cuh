@@ -328,24 +328,20 @@ __device__ __forceinline__ void entry_point64(const FrameDesc &fd, int4 e, doubl
     }
 }
 
-// Escape count of a FP64 slice point, in FP64.  An axis-aligned slice takes the
-// axis form of the first step, whose operations are those of dq_iter on the
-// zero components: the same iterate.
+// One step of the bounds (er, ed) of an orbit's distance from the exact one, from
+// the norms of its halves (see count_bound).  With the dual-number modulus
+// (MOD 1) no test sees the dual half, and the real half does not depend on it.
 template <int SQ, int MOD>
-__device__ __forceinline__ int count64(const FrameDesc &fd, double (&z)[8])
+__device__ __forceinline__ void bound_step(float &er, float &ed, float ar, float ad, float round)
 {
-    return fd.axis_slice ? classify_scalar_axis<double, SQ, MOD>(z, fd.d, fd.max_iter)
-                         : classify_scalar<double, SQ, MOD>(z, fd.d, fd.max_iter);
-}
-
-// FP64 recheck of one queued sample: the pixel is queued for an FP64 re-render
-// when the sample's FP64 escape count differs from its FP32 one.
-template <int SQ, int MOD>
-__device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch &sc, int4 e)
-{
-    double z[8];
-    entry_point64(fd, e, z);
-    if (count64<SQ, MOD>(fd, z) != e.w) mark_dirty(fd, sc, e.x);
+    const float ner = fmaf(er, fmaf(2.f, ar, er), round);
+    if (MOD == 0) {
+        if (SQ == 0)
+            ed = fmaf(2.f, fmaf(ar, ed, fmaf(ad, er, er * ed)), round);
+        else
+            ed = fmaf(ed, fmaf(2.f, ad, ed), round);
+    }
+    er = ner;
 }
 
 // Escape count of a sample by its FP32 orbit beside a bound (er, ed) of that
@@ -370,14 +366,10 @@ __device__ __forceinline__ int count_bound(const FrameDesc &fd, float (&z)[8], f
     float r2 = fmaf(z[0], z[0], sp), d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
     float ar = sqrt_approx(r2), ad = sqrt_approx(d2);
     certain = true;
+#pragma unroll 1
     for (int n = 1; n <= fd.max_iter; ++n) {
-        const float round = 5.6f * u * (r2 + d2 + fd.settle_cn);
-        const float ner = fmaf(er, fmaf(2.f, ar, er), round);
-        if (SQ == 0)
-            ed = fmaf(2.f, fmaf(ar, ed, fmaf(ad, er, er * ed)), round);
-        else
-            ed = fmaf(ed, fmaf(2.f, ad, ed), round);
-        er = ner;
+        const float round = 5.6f * u * ((MOD == 0 ? r2 + d2 : r2) + fd.settle_cn);
+        bound_step<SQ, MOD>(er, ed, ar, ad, round);
         dq_iter<float, SQ, MOD>(z, z, sp, F.c);
         r2 = fmaf(z[0], z[0], sp);
         d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
@@ -417,10 +409,155 @@ __device__ __forceinline__ int count_bound64(const FrameDesc &fd, const double (
     return count_bound<SQ, MOD>(fd, z, e0, e0, certain);
 }
 
+// A sum of products kept in two floats h + l: every product's and every
+// addition's rounding error is computed exactly by FMA and two-sum (Dekker 1971,
+// Knuth) and gathered in l, whose own roundings are of the order u^2 of the
+// terms.
+struct Sum2 {
+    float h, l;
+    __device__ __forceinline__ void add(float p, float e)
+    {
+        // the _rn forms are never contracted into an FMA
+        const float s = __fadd_rn(h, p), b = __fsub_rn(s, h);
+        l += __fadd_rn(__fsub_rn(h, __fsub_rn(s, b)), __fsub_rn(p, b)) + e;
+        h = s;
+    }
+    __device__ __forceinline__ void add_product(float ah, float al, float bh, float bl)
+    {
+        const float p = __fmul_rn(ah, bh);
+        add(p, fmaf(ah, bl, fmaf(al, bh, fmaf(ah, bh, -p))));
+    }
+    __device__ __forceinline__ void store(float &oh, float &ol) const
+    {
+        oh = __fadd_rn(h, l);
+        ol = __fsub_rn(l, __fsub_rn(oh, h));
+    }
+};
+
+// count_bound of a FP64 point with the orbit in two floats per component (about
+// 48 bits): for the samples whose FP32 orbit cannot decide, late orbits and samples next to the
+// surface above all.  A step takes about 260 FP32 instructions, against 27 FP64
+// instructions that hold the FP64 pipe for 1,728 cycles (512 x 512, max_iter 24:
+// recheck pass 0.38 -> 0.18 ms).  The rounding of a step is below 30 u^2 of its
+// terms, the bound takes 128 u^2 of |z_r|^2 + |z_d|^2 + |c|; the modulus needs the high
+// parts only (14 u of itself), unless R^2 lies as close as that.
+template <int SQ, int MOD>
+__device__ __forceinline__ int count_bound2(const FrameDesc &fd, const double (&z64)[8], bool &certain)
+{
+    constexpr float u = 5.9604645e-8f;
+    constexpr int nc = MOD == 0 ? 8 : 4;  // components that a test can see
+    const float R2 = fd.f.R2, hi = R2 * (1.f + 2.f * u), lo = R2 * (1.f - 2.f * u);
+    float zh[8], zl[8];
+#pragma unroll
+    for (int j = 0; j < nc; ++j) {
+        zh[j] = zl[j] = 0.f;
+        if (j < 3 || !fd.axis_slice) {
+            zh[j] = (float)z64[j];
+            zl[j] = (float)(z64[j] - (double)zh[j]);
+        }
+    }
+    auto norms = [&](float &r2, float &d2) {
+        r2 = fmaf(zh[3], zh[3], fmaf(zh[2], zh[2], fmaf(zh[1], zh[1], zh[0] * zh[0])));
+        d2 = MOD == 0 ? fmaf(zh[7], zh[7], fmaf(zh[6], zh[6], fmaf(zh[5], zh[5], zh[4] * zh[4]))) : 0.f;
+    };
+    float r2, d2;
+    norms(r2, d2);
+    float er = 4.f * u * u * (r2 + d2 + 1.f), ed = er;
+    certain = true;
+#pragma unroll 1
+    for (int n = 1; n <= fd.max_iter; ++n) {
+        bound_step<SQ, MOD>(er, ed, sqrt_approx(r2), sqrt_approx(d2), 128.f * u * u * (r2 + d2 + fd.settle_cn));
+        float oh[8], ol[8];
+        // component i starts from c_i
+        auto from_c = [&](int i) {
+            const float ch = fd.f.c[i];
+            return Sum2{ch, (float)(fd.d.c[i] - (double)ch)};
+        };
+        const float t0h = zh[0] + zh[0], t0l = zl[0] + zl[0];
+        {
+            Sum2 a = from_c(0);
+            a.add_product(zh[0], zl[0], zh[0], zl[0]);
+#pragma unroll
+            for (int i = 1; i < 4; ++i) a.add_product(-zh[i], -zl[i], zh[i], zl[i]);
+            a.store(oh[0], ol[0]);
+        }
+#pragma unroll
+        for (int i = 1; i < 4; ++i) {
+            Sum2 a = from_c(i);
+            a.add_product(t0h, t0l, zh[i], zl[i]);
+            a.store(oh[i], ol[i]);
+        }
+        if (MOD == 0) {
+            const float s0h = zh[4] + zh[4], s0l = zl[4] + zl[4];
+            Sum2 a = from_c(4);
+            if (SQ == 0) {
+                a.add_product(t0h, t0l, zh[4], zl[4]);
+#pragma unroll
+                for (int i = 1; i < 4; ++i) a.add_product(-2.f * zh[i], -2.f * zl[i], zh[4 + i], zl[4 + i]);
+            } else {
+                a.add_product(zh[4], zl[4], zh[4], zl[4]);
+#pragma unroll
+                for (int i = 5; i < 8; ++i) a.add_product(-zh[i], -zl[i], zh[i], zl[i]);
+            }
+            a.store(oh[4], ol[4]);
+#pragma unroll
+            for (int i = 5; i < 8; ++i) {
+                Sum2 b = from_c(i);
+                if (SQ == 0) {
+                    b.add_product(t0h, t0l, zh[i], zl[i]);
+                    b.add_product(s0h, s0l, zh[i - 4], zl[i - 4]);
+                } else {
+                    b.add_product(s0h, s0l, zh[i], zl[i]);
+                }
+                b.store(oh[i], ol[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < nc; ++i) {
+            zh[i] = oh[i];
+            zl[i] = ol[i];
+        }
+        norms(r2, d2);
+        const float m = r2 + d2;
+        float dev = er * fmaf(2.f, sqrt_approx(r2), er);
+        if (MOD == 0) dev = fmaf(ed, fmaf(2.f, sqrt_approx(d2), ed), dev);
+        dev = fmaf(1.01f, dev, 14.f * u * m);
+        if (m - dev > hi) return n;
+        if (!(m + dev < lo)) {
+            certain = false;
+            return 0;
+        }
+    }
+    return 0;
+}
+
+// Escape count of a FP64 slice point, as FP64 evaluation gives it: by the
+// two-float orbit where its bound decides, else in FP64.  An axis-aligned
+// slice takes the axis form of the first step, whose operations are those of
+// dq_iter on the zero components: the same iterate.
+template <int SQ, int MOD>
+__device__ __forceinline__ int count64(const FrameDesc &fd, double (&z)[8])
+{
+    bool certain;
+    const int n = count_bound2<SQ, MOD>(fd, z, certain);
+    if (certain) return n;
+    return fd.axis_slice ? classify_scalar_axis<double, SQ, MOD>(z, fd.d, fd.max_iter)
+                         : classify_scalar<double, SQ, MOD>(z, fd.d, fd.max_iter);
+}
+
+// FP64 recheck of one queued sample: the pixel is queued for an FP64 re-render
+// when the sample's FP64 escape count differs from its FP32 one.
+template <int SQ, int MOD>
+__device__ __forceinline__ void recheck_entry(const FrameDesc &fd, const Scratch &sc, int4 e)
+{
+    double z[8];
+    entry_point64(fd, e, z);
+    if (count64<SQ, MOD>(fd, z) != e.w) mark_dirty(fd, sc, e.x);
+}
+
 // Lockstep classification of one sample per lane (classify_lockstep), FP64 by
-// the bound first: a lane whose count the FP32 orbit's bound proves needs no
-// FP64 iteration, and a warp iterates in FP64 only when some lane does.  FP32
-// samples are classified as they are.
+// the bounds first: a lane whose count the FP32 orbit's bound proves needs no
+// more, the others take count64.  FP32 samples are classified as they are.
 template <typename T, int SQ, int MOD, bool RECHECK>
 __device__ __forceinline__ int classify_sample(const FrameDesc &fd, T (&z)[8], bool part, bool &marginal)
 {
@@ -430,11 +567,8 @@ __device__ __forceinline__ int classify_sample(const FrameDesc &fd, T (&z)[8], b
         bool certain = true;
         int n = 1;
         if (part) n = count_bound64<SQ, MOD>(fd, z, certain);
-        const bool again = part && !certain;
-        if (__any_sync(kFull, again)) {
-            const int m = classify_lockstep<T, SQ, MOD, false>(z, fd.d, fd.max_iter, again, marginal);
-            if (again) n = m;
-        }
+        if (part && !certain) n = count64<SQ, MOD>(fd, z);
+        __syncwarp();
         return n;
     } else {
         return classify_lockstep<T, SQ, MOD, RECHECK>(z, frame<T>(fd), fd.max_iter, part, marginal);
@@ -637,6 +771,7 @@ __device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, Tile
             double z[8];
             for (int j = 0; j < 8; ++j) z[j] = F.O[j] + p[0] * F.E[0][j] + p[1] * F.E[1][j] + p[2] * F.E[2][j];
             double sp = dq_sp<double>(z);
+#pragma unroll 1
             for (int n = 0; n < n_star; ++n) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
             its += (unsigned)n_star;
             fv = modulus<double, MOD>(z);
@@ -659,13 +794,11 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
 }
 
 // Recheck entries of one warp are staged in shared memory.  At the end of its
-// tile the warp rechecks them itself (recheck_staged): those whose FP32 count a
-// rounding bound proves are done, the others are evaluated in FP64, which
-// overlaps with the FP32 march of the other warps on the SM instead of running
-// as a pass of its own after the march.  A tile that fills the stage
-// (kQStage entries per warp; a round adds at most 64) appends the staged
-// entries to the frame's queue instead, in one block (one atomic), for the
-// recheck pass.
+// tile the warp drops those whose FP32 count a rounding bound proves
+// (recheck_staged); the others go to the frame's queue for the recheck pass, in
+// blocks of 32 (one atomic).  A tile that fills the stage (kQStage entries per
+// warp; a round adds at most 64) appends the staged entries to the queue as
+// they are.
 constexpr int kQStage = 256;
 // Ray parameter of a half without a sample in the recheck march: its first
 // iterate overflows (modulus +inf) and the later ones are infinite or NaN, so
@@ -698,12 +831,20 @@ __device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch 
     __syncwarp();
 }
 
+// recheck_entry out of line, for entries that find the queue full.
+template <int SQ, int MOD>
+__device__ __noinline__ void recheck_entry_call(const FrameDesc &fd, const Scratch &sc, int4 e)
+{
+    recheck_entry<SQ, MOD>(fd, sc, e);
+}
+
 // Recheck of a warp's staged entries qs[0, qn) (qn warp-uniform), counted as
 // rechecks from entry `counted` on: entries whose FP32 count is certain are done;
-// the others are gathered at the front and rechecked in FP64 in full batches of
-// 32 (an FP64 warp instruction takes the same time for one lane as for 32).
-// Returns how many are left in qs (fewer than 32); they stay staged for the
-// warp's next tile or go to the recheck queue (flush_rest).
+// the others are gathered at the front and appended to the frame's queue 32 at a
+// time, for the recheck pass.  (Evaluating them here put the FP64 and two-float
+// code between a warp's tiles: instruction fetch then stalled the march, 0.76
+// against 0.60 ms at 1080p, 1.51 against 0.97 ms on a random slice.)  Returns how many are left in qs (fewer than 32);
+// they stay staged for the warp's next tile (flush_rest after its last).
 template <int SQ, int MOD, bool AXIS>
 __device__ __forceinline__ int recheck_staged(const FrameDesc &fd, const Scratch &sc, int4 *qs, int qn, int counted)
 {
@@ -725,7 +866,14 @@ __device__ __forceinline__ int recheck_staged(const FrameDesc &fd, const Scratch
         __syncwarp();
         if (out >= 32) {  // fewer than 32 were left, at most 32 came: one batch
             out -= 32;
-            recheck_entry<SQ, MOD>(fd, sc, qs[out + lane]);
+            const int4 v = qs[out + lane];
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&sc.ctr->queue_count, 32u);
+            at = __shfl_sync(kFull, at, 0) + lane;
+            if (at < sc.queue_cap)
+                sc.queue[at] = v;
+            else
+                recheck_entry_call<SQ, MOD>(fd, sc, v);
             __syncwarp();
         }
     }
@@ -967,22 +1115,26 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     const FrameT<float> &F = fd.f;
     const int lane = threadIdx.x & 31;
     const int N = fd.N, max_iter = fd.max_iter;
-    const int tx = (int)(tile % (unsigned)fd.tiles_x), ty = (int)(tile / (unsigned)fd.tiles_x);
-    auto px = [&](int slot) { return tx * fd.tile_w + slot % fd.tile_w; };
-    auto py = [&](int slot) { return ty * fd.tile_h + slot / fd.tile_w; };
-    int pixa = 0, pixb = 0, xya = 0, xyb = 0;
+    // pixels of the tile slots `lane` and `lane + 32`, x | y << 16 (no division
+    // at the end of the tile, where they are needed again)
+    int xya, xyb;
+    {
+        const int ty = (int)(tile / (unsigned)fd.tiles_x), tx = (int)tile - ty * fd.tiles_x;
+        const int sya = lane / fd.tile_w, syb = (lane + 32) / fd.tile_w;
+        xya = (tx * fd.tile_w + lane - sya * fd.tile_w) | ((ty * fd.tile_h + sya) << 16);
+        xyb = (tx * fd.tile_w + lane + 32 - syb * fd.tile_w) | ((ty * fd.tile_h + syb) << 16);
+    }
+    const int xa = xya & 0xffff, ya = xya >> 16, xb = xyb & 0xffff, yb = xyb >> 16;
+    int pixa = 0, pixb = 0;
     bool acta, actb, skipa = false, skipb = false;
     // as in march2_tile: zeta_0 = A + t D on an axis slice, else the first
     // iterate Q0 + s (Q1 + s Q2) with Q0 in D and s = t + dot
     float2 D[AXIS ? 3 : 8], tin, dl;
     float2 Q1[AXIS ? 1 : 8], Q2[AXIS ? 1 : 8];
     {
-        const int xa = px(lane), ya = py(lane), xb = px(lane + 32), yb = py(lane + 32);
         if (RECHECK) {
             pixa = ya * fd.W + xa;
             pixb = yb * fd.W + xb;
-            xya = xa | (ya << 16);
-            xyb = xb | (yb << 16);
         }
         const bool va = xa < fd.W && ya < fd.H, vb = xb < fd.W && yb < fd.H;
         float da[3] = {0.f, 0.f, 1.f}, db[3] = {0.f, 0.f, 1.f};
@@ -1154,7 +1306,6 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     const bool hita = kfa >= 0, hitb = kfb >= 0;
     const int nesca = (hita ? kfa : k1) - k0, nescb = (hitb ? kfb : k1) - k0;
     if constexpr (SPLIT) {  // this range's partial result per ray (see march_merge_kernel)
-        const int xa = px(lane), ya = py(lane), xb = px(lane + 32), yb = py(lane + 32);
         const unsigned r = (unsigned)(kb / fd.k_chunk);
         const int64_t npx = (int64_t)fd.W * fd.H, base = (int64_t)r * npx;
         if (xa < fd.W && ya < fd.H && !skipa) {
@@ -1174,7 +1325,6 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     st.iters += (boxa ? suma + nesca : 0) + (boxb ? sumb + nescb : 0);
     st.samples += (boxa ? nesca + (hita ? 1 : 0) : 0) + (boxb ? nescb + (hitb ? 1 : 0) : 0);
     st.hits += (hita ? 1 : 0) + (hitb ? 1 : 0);
-    const int xa = px(lane), ya = py(lane), xb = px(lane + 32), yb = py(lane + 32);
     const bool va = xa < fd.W && ya < fd.H, vb = xb < fd.W && yb < fd.H;
     if (va && !hita) write_miss<float>(fd, xa, ya, boxa ? maxa + 1 : 0);
     if (vb && !hitb) write_miss<float>(fd, xb, yb, boxb ? maxb + 1 : 0);
@@ -1205,6 +1355,7 @@ __device__ __forceinline__ void normal_shade(const FrameDesc &fd, const FrameT<T
 #pragma unroll
             for (int i = 0; i < 8; ++i) z[i] = dfma(hs, F.E[a][i], dfma(depth, D[i], F.A[i]));
             T sp = dq_sp<T>(z);
+#pragma unroll 1
             for (int n = 0; n < nmax; ++n)
                 if (n < n_star) dq_iter<T, SQ, MOD>(z, z, sp, F.c);
             fv[s] = modulus<T, MOD>(z);
@@ -1255,6 +1406,7 @@ __device__ __forceinline__ void late_normals(const FrameDesc &fd, unsigned mask,
 #pragma unroll
         for (int i = 0; i < 8; ++i) z[i] = fma(hs, F.E[a][i], fma(t, D[i], F.A[i]));
         double sp = dq_sp<double>(z);
+#pragma unroll 1
         for (int n = 0; n < nmax; ++n)
             if (n < ns) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
         const double fv = modulus<double, MOD>(z);
@@ -1386,6 +1538,7 @@ __device__ __forceinline__ void group_normal(const FrameDesc &fd, const FrameT<U
         for (int i = 0; i < 8; ++i) z[i] = dfma(hs, F.E[a][i], dfma(depth, D[i], F.A[i]));
         U sp = dq_sp<U>(z);
         const int ns = part && q < 6 ? n_lo : 0;
+#pragma unroll 1
         for (int n = 0; n < nmax; ++n)
             if (n < ns) dq_iter<U, SQ, MOD>(z, z, sp, F.c);
         const U fv = modulus<U, MOD>(z);

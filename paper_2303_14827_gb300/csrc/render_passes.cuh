@@ -201,9 +201,12 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 5 : 4)  // the general form kee
 
 // march2_kernel with two samples of each ray per round (march4_tile).  Its
 // four sets of iterates take more registers: four CTAs per SM on an axis
-// slice, three with the general form's first-iterate coefficients.
+// slice, three with the general form's first-iterate coefficients.  The recheck
+// form with settled blocks takes three too: at four it spilled, and 16 warps at
+// as many places of its longer code stalled on instruction fetch (recheck march
+// at 1080p 0.562 / 0.525 ms at four / three).
 template <int SQ, int MOD, bool RECHECK, bool AXIS, bool SETTLE>
-__global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_kernel(const __grid_constant__ FrameDesc fd,
+__global__ void __launch_bounds__(kBlock, AXIS && !(RECHECK && SETTLE) ? 4 : 3) march4_kernel(const __grid_constant__ FrameDesc fd,
                                                                       const Scratch sc)
 {
     __shared__ int4 stage[RECHECK ? kBlock / 32 : 1][RECHECK ? kQStage : 1];  // recheck entries, per warp

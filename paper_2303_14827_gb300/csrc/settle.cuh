@@ -53,10 +53,12 @@ __device__ __forceinline__ float warp_max(float v)
     asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
     return r;
 }
+// Square root to 1e-6 relative; arguments below 1e-38 count as zero, which the
+// bounds' additive rounding terms cover.
 __device__ __forceinline__ float sqrt_approx(float v)
 {
     float r;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
     return r;
 }
 
@@ -155,6 +157,7 @@ __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[
     }
     const int cap = min(kSettleCap, fd.max_iter);
     const float2 two = make_float2(2.f, 2.f), neg = make_float2(-1.f, -1.f), one_two = make_float2(1.f, 2.f);
+#pragma unroll 1
     for (int n = 1; n <= cap; ++n) {
         // the remainder, from the norms of this step's set
         {
@@ -291,6 +294,7 @@ __device__ __forceinline__ unsigned settle_chunk(const FrameDesc &fd, const Tile
     const int lane = threadIdx.x & 31;
     const float inv_n = 1.f / (float)fd.N;
     unsigned w = 0, todo = 0;
+#pragma unroll 1
     for (bool whole = true;; whole = false) {
         int ka, kb, src = -1;
         bool valid;
