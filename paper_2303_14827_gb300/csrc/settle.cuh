@@ -29,6 +29,7 @@
 namespace dqj {
 
 constexpr int kSettleCap = 6;     // deepest escape step proved: deeper shells are thinner than a pair of samples
+constexpr int kSettleInside = 15; // count of a box without an escape (settle_box<INSIDE>)
 constexpr int kSettlePairs = 8;   // sample pairs per block at most
 constexpr int kSettleChunk = 32 * 2 * kSettlePairs;  // samples settled at a time by a warp
 constexpr int kSettleMin = 8;     // chunks of this many samples or fewer are marched outright
@@ -122,10 +123,11 @@ __device__ __forceinline__ void block_box(const TileBox &B, float inv_n, int ka,
 }
 
 // The escape count shared by every sample of the box (p, h), or 0 when it is
-// not proved.  The centre and the first generator advance in the halves of u,
+// not proved.  INSIDE: counts to 14, and 15 when no sample of the box escapes by
+// max_iter.  The centre and the first generator advance in the halves of u,
 // the other two generators in those of v.  AXIS: components 3..7 of the slice
 // are zero, so the first step needs only components 0..2.
-template <int SQ, int MOD, bool AXIS>
+template <int SQ, int MOD, bool AXIS, bool INSIDE = false>
 __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[3], const float (&h)[3], float rho,
                                           float e1)
 {
@@ -155,7 +157,7 @@ __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[
         ar = sqrt_approx(r);
         ad = AXIS ? 0.f : sqrt_approx(d);
     }
-    const int cap = min(kSettleCap, fd.max_iter);
+    const int cap = INSIDE ? fd.max_iter : min(kSettleCap, fd.max_iter);
     const float2 two = make_float2(2.f, 2.f), neg = make_float2(-1.f, -1.f), one_two = make_float2(1.f, 2.f);
 #pragma unroll 1
     for (int n = 1; n <= cap; ++n) {
@@ -275,10 +277,10 @@ __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[
             }
         }
         dev = fmaf(2.0004f, dev, 1e-5f * (m + sq));
-        if (m - dev > hi) return n;
+        if (m - dev > hi) return !INSIDE || n < kSettleInside ? n : 0;
         if (!(fmaf(1.0002f, sq, m + dev) < lo)) return 0;
     }
-    return 0;
+    return INSIDE ? kSettleInside : 0;
 }
 
 // Settled counts of the samples [kc, ke) of a tile, ke - kc <= kSettleChunk, in

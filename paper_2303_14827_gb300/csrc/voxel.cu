@@ -3,15 +3,19 @@
 // like a ray sample (slice map, then the escape-time iteration), giving an
 // occupancy byte (1 = no escape by max_iter) and the escape count.
 //
-// Work unit of the FP32 kernel: a 32 x 2 segment (x = x0 .. x0+31 in rows
-// 2 jp and 2 jp + 1 of slice k).  The rows' slice images of (0, y, z) are
-// warp-uniform; each lane advances its column's two cells in float2 halves
-// with the paired march classification, so a cell costs the same arithmetic
-// as a march sample.  Warps claim segments through an atomic counter
-// (persistent grid).
+// Fine grids (FP32) are taken in bricks of 16 x 8 x 4 cells, eight sub-bricks of 8 x
+// 4 x 2 each.  Far from the set the escape count is constant over whole bricks, and a
+// bound proves it (settle_box): those are filled, as are the settled sub-bricks
+// of the others; only what is left is classified, a sub-brick at a time (lane =
+// column, its two z cells in the float2 halves of the paired march
+// classification).  Coarse grids classify every cell, in 32 x 2 row segments.
+// Warps claim their work through an atomic counter (persistent grid).
 // FP64 runs one cell per lane; FP32 + recheck queues cells whose modulus came
 // within the margin of R^2 and re-classifies them in FP64 afterwards (a queue
 // overflow re-runs the whole grid in FP64).
+#include <algorithm>
+#include <cmath>
+
 #include "render_common.cuh"
 #include "runtime.h"
 
@@ -21,8 +25,12 @@ namespace {
 
 struct VoxelArgs {
     int32_t g;
-    uint32_t segs_per_row;
+    uint32_t segs_per_row;                 // FP32, row segments
     uint64_t nsegs;
+    uint32_t bricks_x, bricks_y, nbricks;  // FP32, bricks along x, along y, in all
+    uint32_t per_claim;                    // bricks claimed at a time, 1..32
+    float radius;                          // |slice origin| + largest |corner| of the box
+    int32_t wide;                          // rows of 16 cells are 16-byte aligned in occ and counts
     uint8_t *occ;       // g^3 or NULL
     uint16_t *count;    // g^3 or NULL
     Counters *ctr;      // stats in DQJ_STAT_* order, tile_next = segment claim, queue_count
@@ -72,7 +80,8 @@ __device__ __forceinline__ long long fix_cell(const VoxelArgs &va, uint64_t lin,
 // advance incrementally (no division per segment).
 constexpr uint32_t kBatch = 16;
 
-// Paired FP32 classification of two cells per lane.  A segment is 32 x 2
+// Grids of fewer than kBrickGrid cells a side: paired FP32 classification of two
+// cells per lane, every cell.  A segment is 32 x 2
 // cells: 32 along x in the row pair (2 jp, 2 jp + 1) of one z slice; lane l
 // takes column x0 + l of both rows, so its two cells share px and differ only
 // in the rows' (warp-uniform) slice bases, and each warp store covers 32
@@ -179,6 +188,209 @@ __global__ void __launch_bounds__(kBlock, 5) voxel2_kernel(const __grid_constant
     if (RECHECK) flush_stat(&va.ctr->stats[4], rechecks);
 }
 
+// Bricks against 32 x 2 row segments, FP32, axis / random slice (ms): 256^3 0.105 /
+// 0.143 against 0.092 / 0.135, 300^3 0.141 / 0.192 against 0.130 / 0.199, 333^3 0.166 /
+// 0.225 against 0.166 / 0.253, 400^3 0.19 / 0.29 against 0.25 / 0.40, 1024^3 1.97 /
+// 2.95 against 3.42 / 5.73: coarse bricks settle too seldom to pay for the bound.
+constexpr int kBrickGrid = 336;
+constexpr int kBrickX = 16, kBrickY = 8, kBrickZ = 4;  // a brick; its eight sub-bricks are half as long each way
+
+// The count (15: inside) shared by the cells [x, x + nx) x [y, y + ny) x [z, z + nz) (clipped to
+// the grid), or 0 when the bound does not prove one.
+template <int SQ, int MOD, bool AXIS>
+__device__ __forceinline__ int settle_cells(const FrameDesc &fd, const VoxelArgs &va, const float (&step)[3], int x,
+                                            int y, int z, int nx, int ny, int nz)
+{
+    const int lo[3] = {x, y, z}, n[3] = {min(nx, va.g - x), min(ny, va.g - y), min(nz, va.g - z)};
+    const float rho = 4e-6f * va.radius, e1 = 8e-6f * va.radius * va.radius;
+    float p[3], h[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        p[a] = fmaf((float)lo[a] + 0.5f * (float)n[a], step[a], fd.f.bmin[a]);
+        h[a] = fmaf(0.5f * (float)(n[a] - 1), step[a], rho);
+    }
+    return settle_box<SQ, MOD, AXIS, true>(fd, p, h, rho, e1);
+}
+
+// A row of 16 settled cells starting at lin.
+__device__ __forceinline__ void fill_row16(const VoxelArgs &va, uint32_t lin, int n)
+{
+    const bool in = n == kSettleInside;
+    const unsigned o = in ? 0x01010101u : 0u, v = in ? 0u : (unsigned)n * 0x10001u;
+    if (va.occ) *reinterpret_cast<uint4 *>(va.occ + lin) = make_uint4(o, o, o, o);
+    if (va.count) {
+        uint4 *c = reinterpret_cast<uint4 *>(va.count + lin);
+        c[0] = make_uint4(v, v, v, v);
+        c[1] = make_uint4(v, v, v, v);
+    }
+}
+
+// Grids of kBrickGrid cells a side or more (see the head of this file).  A claim's bricks are
+// settled one per lane, then the sub-bricks of the bricks left over, four bricks
+// at a time; lane b's word holds the counts of brick b's sub-bricks, four bits
+// each.  1024^3 (default constant): nine in ten sub-bricks settle
+// (inside ones too), 3.42 -> 1.97 ms; the 3.2 GB written take 0.47 ms at the
+// measured copy rate.  What is left is the classification of the others, whose
+// cells run 8 to max_iter steps.
+template <int SQ, int MOD, bool RECHECK, bool AXIS>
+__global__ void __launch_bounds__(kBlock, 5) voxel_brick_kernel(const __grid_constant__ FrameDesc fd, const VoxelArgs va)
+{
+    const FrameT<float> &F = fd.f;
+    const int lane = threadIdx.x & 31;
+    const int g = va.g;
+    const uint32_t gu = (uint32_t)g;
+    const uint32_t max_iter = (uint32_t)fd.max_iter;
+    float step[3];
+    grid_step<float>(F, g, step);
+    const int lx = lane & 7, ly = lane >> 3;  // column of a sub-brick
+    unsigned long long iters = 0, inside_n = 0, rechecks = 0, cells = 0;
+    for (;;) {
+        uint32_t first = 0;
+        if (lane == 0) first = atomicAdd(&va.ctr->tile_next, va.per_claim);
+        first = __shfl_sync(kFull, first, 0);
+        if (first >= va.nbricks) break;
+        const int nb = (int)min(va.per_claim, va.nbricks - first);
+        // lane b: brick first + b
+        int bx, by, bz;
+        {
+            const uint32_t id = first + (uint32_t)min(lane, nb - 1), row = id / va.bricks_x;
+            bx = (int)(id - row * va.bricks_x) * kBrickX;
+            bz = (int)(row / va.bricks_y);
+            by = (int)(row - (uint32_t)bz * va.bricks_y) * kBrickY;
+            bz *= kBrickZ;
+        }
+        unsigned w = 0;
+        {
+            int n = 0;
+            // (a few bricks go to their sub-bricks at once)
+            if (lane < nb && va.per_claim > 4) n = settle_cells<SQ, MOD, AXIS>(fd, va, step, bx, by, bz, kBrickX, kBrickY, kBrickZ);
+            __syncwarp();
+            w = (unsigned)n * 0x11111111u;
+            unsigned todo = __ballot_sync(kFull, lane < nb && n == 0);
+            while (todo) {
+                int blk = -1, src = -1;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int bj = todo ? __ffs(todo) - 1 : -1;
+                    todo &= todo - 1;
+                    if ((lane >> 3) == j) blk = bj;
+                    if (lane == bj) src = 8 * j;
+                }
+                const int from = blk < 0 ? 0 : blk, sb = lane & 7;
+                const int x = __shfl_sync(kFull, bx, from) + (sb & 1) * (kBrickX / 2);
+                const int y = __shfl_sync(kFull, by, from) + (sb >> 1 & 1) * (kBrickY / 2);
+                const int z = __shfl_sync(kFull, bz, from) + (sb >> 2) * (kBrickZ / 2);
+                int m = 0;
+                if (blk >= 0 && x < g && y < g && z < g)
+                    m = settle_cells<SQ, MOD, AXIS>(fd, va, step, x, y, z, kBrickX / 2, kBrickY / 2, kBrickZ / 2);
+                __syncwarp();
+                unsigned v = (unsigned)m << (4 * sb);
+                v |= __shfl_xor_sync(kFull, v, 1);
+                v |= __shfl_xor_sync(kFull, v, 2);
+                v |= __shfl_xor_sync(kFull, v, 4);
+                const unsigned t = __shfl_sync(kFull, v, src < 0 ? 0 : src);
+                if (src >= 0) w = t;
+            }
+        }
+        uint32_t it32 = 0, in32 = 0, cl32 = 0, re32 = 0;
+        for (int b = 0; b < nb; ++b) {
+            const unsigned word = __shfl_sync(kFull, w, b);
+            const int x0 = __shfl_sync(kFull, bx, b), y0 = __shfl_sync(kFull, by, b), z0 = __shfl_sync(kFull, bz, b);
+            const int n0 = (int)(word & 15u);
+            if (va.wide && n0 && word == (unsigned)n0 * 0x11111111u && x0 + kBrickX <= g) {
+                // a settled brick: 32 rows of 16 cells, one per lane
+                const int y = y0 + (lane & 7), z = z0 + (lane >> 3);
+                if (y < g && z < g) {
+                    fill_row16(va, ((uint32_t)z * gu + (uint32_t)y) * gu + (uint32_t)x0, n0);
+                    it32 += 16u * (n0 == kSettleInside ? max_iter : (uint32_t)n0);
+                    in32 += n0 == kSettleInside ? 16u : 0u;
+                    cl32 += 16u;
+                }
+                continue;
+            }
+            // the lane's column in the brick's first sub-brick, its coordinates in
+            // cells (exact: no conversion per sub-brick) and linear index
+            const int xb = x0 + lx, yb = y0 + ly;
+            const float xf = (float)xb + 0.5f, yf = (float)yb + 0.5f, zf = (float)z0 + 0.5f;
+            const uint32_t lin = ((uint32_t)z0 * gu + (uint32_t)yb) * gu + (uint32_t)xb;
+#pragma unroll 1
+            for (int sb = 0; sb < 8; ++sb) {
+                const int dx = (sb & 1) * (kBrickX / 2), dy = (sb >> 1 & 1) * (kBrickY / 2), dz = (sb >> 2) * (kBrickZ / 2);
+                const int z = z0 + dz;
+                if (x0 + dx >= g || y0 + dy >= g || z >= g) continue;  // warp-uniform
+                const int n = (int)((word >> (4 * sb)) & 15u);
+                const bool va_ = xb + dx < g && yb + dy < g, vb_ = va_ && z + 1 < g;
+                const uint32_t la = lin + ((uint32_t)dz * gu + (uint32_t)dy) * gu + (uint32_t)dx, lb = la + gu * gu;
+                cl32 += (va_ ? 1u : 0u) + (vb_ ? 1u : 0u);
+                if (n) {  // a settled sub-brick
+                    const bool in = n == kSettleInside;
+                    const uint32_t c = (va_ ? 1u : 0u) + (vb_ ? 1u : 0u);
+                    if (va_) write_cell(va, la, in, n);
+                    if (vb_) write_cell(va, lb, in, n);
+                    it32 += (in ? max_iter : (uint32_t)n) * c;
+                    in32 += in ? c : 0u;
+                    continue;
+                }
+                bool aa = va_, ab = vb_;
+                const float px = fmaf(xf + (sb & 1 ? (float)(kBrickX / 2) : 0.f), step[0], F.bmin[0]);
+                const float py = fmaf(yf + (sb & 2 ? (float)(kBrickY / 2) : 0.f), step[1], F.bmin[1]);
+                const float zc = zf + (sb & 4 ? (float)(kBrickZ / 2) : 0.f);
+                const float pz = fmaf(zc, step[2], F.bmin[2]), pz1 = fmaf(zc + 1.f, step[2], F.bmin[2]);
+                float2 q[8];
+#pragma unroll
+                for (int i = 0; i < (AXIS ? 3 : 8); ++i) {  // AXIS: components 3..7 are zero
+                    const float r = fmaf(py, F.E[1][i], F.O[i]);
+                    q[i] = f2fma(make_float2(px, px), make_float2(F.E[0][i], F.E[0][i]),
+                                 make_float2(fmaf(pz, F.E[2][i], r), fmaf(pz1, F.E[2][i], r)));
+                }
+                int ca, cb;
+                bool live;
+                float2 dm;
+                classify_lockstep2<SQ, MOD, RECHECK, AXIS>(q, fd.p2, F.R2, fd.max_iter, aa, ab, ca, cb, dm, live);
+                const bool mga = dm.x <= fd.p2.margin_t, mgb = dm.y <= fd.p2.margin_t;
+                if (va_) {
+                    write_cell(va, la, aa, ca + 1);
+                    it32 += aa ? max_iter : (uint32_t)(ca + 1);
+                    in32 += aa ? 1u : 0u;
+                }
+                if (vb_) {
+                    write_cell(va, lb, ab, cb + 1);
+                    it32 += ab ? max_iter : (uint32_t)(cb + 1);
+                    in32 += ab ? 1u : 0u;
+                }
+                if (RECHECK) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const bool push = h == 0 ? (va_ && mga) : (vb_ && mgb);
+                        const unsigned m = __ballot_sync(kFull, push);
+                        if (m == 0) continue;
+                        const int leader = __ffs(m) - 1;
+                        unsigned at = 0;
+                        if (lane == leader) at = atomicAdd(&va.ctr->queue_count, (unsigned)__popc(m));
+                        at = __shfl_sync(kFull, at, leader);
+                        if (push) {
+                            const unsigned slot = at + __popc(m & ((1u << lane) - 1u));
+                            if (slot < va.queue_cap)
+                                va.queue[slot] = h == 0 ? la : lb;
+                            else
+                                atomicAdd(&va.ctr->stats[7], 1ull);  // overflow: the FP64 pass re-runs the grid
+                            re32 += 1;
+                        }
+                    }
+                }
+            }
+        }
+        iters += it32;
+        inside_n += in32;
+        cells += cl32;
+        rechecks += re32;
+    }
+    flush_stat(&va.ctr->stats[0], iters);
+    flush_stat(&va.ctr->stats[2], cells);
+    flush_stat(&va.ctr->stats[3], inside_n);
+    if (RECHECK) flush_stat(&va.ctr->stats[4], rechecks);
+}
+
 // FP64 classification, one cell per lane (32-cell row segments).
 template <int SQ, int MOD>
 __global__ void __launch_bounds__(kBlock) voxel64_kernel(const __grid_constant__ FrameDesc fd, const VoxelArgs va)
@@ -208,7 +420,7 @@ __global__ void __launch_bounds__(kBlock) voxel64_kernel(const __grid_constant__
             for (int i = 0; i < 8; ++i) z[i] = fma(p0, F.E[0][i], base[i]);
             bool mg;
             const bool part = x < g;
-            const int n = classify_lockstep<double, SQ, MOD, false>(z, F, fd.max_iter, part, mg);
+            const int n = classify_sample<double, SQ, MOD, false>(fd, z, part, mg);
             if (part) {
                 write_cell(va, (uint64_t)row * (uint64_t)g + x, n == 0, n);
                 iters += n ? (unsigned)n : (unsigned)fd.max_iter;
@@ -235,7 +447,9 @@ __device__ __forceinline__ int cell_fp64(const FrameDesc &fd, int g, uint64_t li
     const double p0 = fma((double)x + 0.5, step[0], F.bmin[0]);
 #pragma unroll
     for (int i = 0; i < 8; ++i) z[i] = fma(p0, F.E[0][i], base[i]);
-    const int n = classify_scalar<double, SQ, MOD>(z, F, fd.max_iter);
+    bool certain;
+    int n = count_bound64<SQ, MOD>(fd, z, certain);
+    if (!certain) n = count64<SQ, MOD>(fd, z);
     it += n ? (unsigned)n : (unsigned)fd.max_iter;
     return n;
 }
@@ -272,28 +486,44 @@ __global__ void __launch_bounds__(kBlock) voxel_overflow_kernel(const __grid_con
 }
 
 template <int SQ, int MOD>
-cudaError_t launch_voxels_t(const FrameDesc &fd, const VoxelArgs &va, cudaStream_t st, int num_sms)
+cudaError_t launch_voxels_t(const FrameDesc &fd, const VoxelArgs &args, cudaStream_t st, int num_sms)
 {
-    static std::atomic<int> g64{0}, g2{0}, gre{0}, gov{0};
+    static std::atomic<int> g64{0}, g2{0}, gb{0}, gre{0}, gov{0};
     if (fd.precision == DQJ_FP64) {
-        voxel64_kernel<SQ, MOD><<<num_sms * resident_per_sm(g64, voxel64_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, va);
+        voxel64_kernel<SQ, MOD><<<num_sms * resident_per_sm(g64, voxel64_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, args);
         return cudaGetLastError();
     }
     const bool re = fd.precision == DQJ_FP32_RECHECK;
-    const int gm = (int)min((uint64_t)num_sms * resident_per_sm(g2, voxel2_kernel<SQ, MOD, false, false>),
-                            (va.nsegs + 4 * kBatch - 1) / (4 * kBatch));
-    const int gg = gm > 0 ? gm : 1;
-    if (re) {
-        if (fd.axis_slice)
-            voxel2_kernel<SQ, MOD, true, true><<<gg, kBlock, 0, st>>>(fd, va);
+    const int axis = fd.axis_slice ? 1 : 0;
+    if (args.g >= kBrickGrid && march_settles()) {
+        // bricks per claim: 32 or 16 (one settle pass of a warp) where every resident
+        // warp gets several claims of that, else four (one pass over their sub-bricks)
+        VoxelArgs va = args;
+        const uint32_t warps =
+            (uint32_t)num_sms * (uint32_t)resident_per_sm(gb, voxel_brick_kernel<SQ, MOD, false, false>) * 4u;
+        va.per_claim = va.nbricks >= 256u * warps ? 32u : va.nbricks >= 64u * warps ? 16u : 4u;
+        const uint32_t claims = (va.nbricks + va.per_claim - 1u) / va.per_claim;
+        const int gg = (int)std::min(warps / 4u, (claims + 3u) / 4u);
+        if (re)
+            axis ? voxel_brick_kernel<SQ, MOD, true, true><<<gg, kBlock, 0, st>>>(fd, va)
+                 : voxel_brick_kernel<SQ, MOD, true, false><<<gg, kBlock, 0, st>>>(fd, va);
         else
-            voxel2_kernel<SQ, MOD, true, false><<<gg, kBlock, 0, st>>>(fd, va);
-        voxel_recheck_kernel<SQ, MOD><<<num_sms * resident_per_sm(gre, voxel_recheck_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, va);
-        voxel_overflow_kernel<SQ, MOD><<<num_sms * resident_per_sm(gov, voxel_overflow_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, va);
-    } else if (fd.axis_slice) {
-        voxel2_kernel<SQ, MOD, false, true><<<gg, kBlock, 0, st>>>(fd, va);
+            axis ? voxel_brick_kernel<SQ, MOD, false, true><<<gg, kBlock, 0, st>>>(fd, va)
+                 : voxel_brick_kernel<SQ, MOD, false, false><<<gg, kBlock, 0, st>>>(fd, va);
     } else {
-        voxel2_kernel<SQ, MOD, false, false><<<gg, kBlock, 0, st>>>(fd, va);
+        const int gm = (int)min((uint64_t)num_sms * resident_per_sm(g2, voxel2_kernel<SQ, MOD, false, false>),
+                                (args.nsegs + 4 * kBatch - 1) / (4 * kBatch));
+        const int gg = gm > 0 ? gm : 1;
+        if (re)
+            axis ? voxel2_kernel<SQ, MOD, true, true><<<gg, kBlock, 0, st>>>(fd, args)
+                 : voxel2_kernel<SQ, MOD, true, false><<<gg, kBlock, 0, st>>>(fd, args);
+        else
+            axis ? voxel2_kernel<SQ, MOD, false, true><<<gg, kBlock, 0, st>>>(fd, args)
+                 : voxel2_kernel<SQ, MOD, false, false><<<gg, kBlock, 0, st>>>(fd, args);
+    }
+    if (re) {
+        voxel_recheck_kernel<SQ, MOD><<<num_sms * resident_per_sm(gre, voxel_recheck_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, args);
+        voxel_overflow_kernel<SQ, MOD><<<num_sms * resident_per_sm(gov, voxel_overflow_kernel<SQ, MOD>), kBlock, 0, st>>>(fd, args);
     }
     return cudaGetLastError();
 }
@@ -346,8 +576,21 @@ extern "C" dqj_status dqj_voxelize(dqj_ctx *ctx, const dqj_params *p, int32_t gr
         derive_frame(*p, fd, 8, 8);
         VoxelArgs va{};
         va.g = grid_n;
-        va.segs_per_row = (uint32_t)((grid_n + 31) / 32);  // 32 x 2 segments of the FP32 kernel
+        va.segs_per_row = (uint32_t)((grid_n + 31) / 32);  // 32 x 2 segments
         va.nsegs = (uint64_t)grid_n * (uint64_t)((grid_n + 1) / 2) * va.segs_per_row;
+        va.bricks_x = (uint32_t)((grid_n + kBrickX - 1) / kBrickX);
+        va.bricks_y = (uint32_t)((grid_n + kBrickY - 1) / kBrickY);
+        va.nbricks = va.bricks_x * va.bricks_y * (uint32_t)((grid_n + kBrickZ - 1) / kBrickZ);
+        double corner = 0.0;
+        for (int a = 0; a < 3; ++a) {
+            const double m = std::max(std::fabs(p->box_min[a]), std::fabs(p->box_max[a]));
+            corner += m * m;
+        }
+        double origin = 0.0;
+        for (int i = 0; i < 8; ++i) origin += p->slice_origin[i] * p->slice_origin[i];
+        va.radius = (float)(std::sqrt(corner) + std::sqrt(origin));
+        va.wide = grid_n % 16 == 0 && (reinterpret_cast<uintptr_t>(occupancy) & 15u) == 0 &&
+                  (reinterpret_cast<uintptr_t>(counts) & 15u) == 0;
         va.occ = occupancy;
         va.count = counts;
         va.ctr = static_cast<Counters *>(ctx->vox_scratch);

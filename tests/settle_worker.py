@@ -61,6 +61,23 @@ def main(path):
             o = r.render(s)
             for k in ("iter", "depth", "normal", "rgba", "stats"):
                 out[f"{i}_{k}"] = o[k].cpu().numpy()
+        # voxel grids: edges of bricks and sub-bricks, rows with and without wide stores
+        rng = np.random.default_rng(32)
+        for i, g in enumerate((64, 71, 100, 336, 337, 345, 352)):
+            for prec in (0, 1, 2) if g <= 100 else (0, 1):
+                s = scenes.default_scene(precision=prec, max_iter=14, c=scenes.random_c(rng))
+                if i % 2:
+                    s["slice_basis"] = scenes.random_slice_frame(rng)
+                occ = torch.full((g ** 3,), 7, dtype=torch.uint8, device="cuda")
+                cnt = torch.full((g ** 3,), 7, dtype=torch.int16, device="cuda")
+                st = torch.zeros(binding.DQJ_NSTATS, dtype=torch.int64, device="cuda")
+                binding.dqj_voxelize(r.ctx, s, g, occ, cnt, st, torch.cuda.current_stream().cuda_stream)
+                tag = f"voxel{g}p{prec}"
+                planes = torch.arange(g ** 3, device="cuda") % 8191 + 1  # weights: a grid as a few sums
+                out[tag + "_iter"] = np.array([int(occ.sum()), int((occ.long() * planes).sum())])
+                out[tag + "_count"] = np.array([int(cnt.sum()), int((cnt.long() * planes).sum())])
+                st[4:7] = 0  # how many cells were rechecked depends on the cells that share a warp's steps
+                out[tag + "_stats"] = st.cpu().numpy()
         torch.cuda.synchronize()
     np.savez(path, **out)
 
