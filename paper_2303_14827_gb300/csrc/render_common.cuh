@@ -634,30 +634,128 @@ __device__ __forceinline__ bool count_certain(const FrameDesc &fd, int x, int y,
     return certain && n == n32;
 }
 
-// Re-render of one pixel by one warp (all 32 lanes call), with the oracle's
-// formulas for the sample positions (the reference sequence of steps) in FP64;
-// a march or bisection sample is classified in FP32 where the rounding bound
-// decides (count_bound), else in FP64; the bisection runs
-// five levels per round across the lanes; the normal is FP64.  The lanes classify 32 consecutive march samples at a time; a ballot
-// finds the first inside one and warp reductions give the largest escape count
-// before it, so the result and the iteration count are those of the
-// sample-by-sample loop.  Bisection runs on every lane alike; the six normal
-// evaluations run on lanes 0..5.  Adds the iterations to its (per lane) and the
-// pixel to npx (lane 0).
-template <int SQ, int MOD>
-__device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, TileBox &box, unsigned long long &its,
-                                            unsigned long long &npx)
+// A hit whose normal is evaluated in FP64: pixel x | y << 16, n*, FP64 depth.
+__device__ __forceinline__ int4 late_hit(int x, int y, int n_star, double depth)
+{
+    const long long b = __double_as_longlong(depth);
+    return make_int4(x | (y << 16), n_star, (int)(unsigned)(b & 0xffffffffll), (int)(b >> 32));
+}
+
+constexpr int kLateGroup = 5;  // hits whose normals a warp evaluates together, six lanes each
+
+// FP64 normals and shading of late hits list[0, count), count <= 5 (all 32 lanes
+// call): the six field evaluations of a hit on six lanes, on the hit's FP64 ray.
+// An FP64 warp instruction takes the same time for one lane as for 32, so
+// evaluating them on the hits' own lanes, or one hit at a time, wasted the
+// others (512 x 512, max_iter 24, 55 % of the hits late: bisection pass 0.74 -> 0.63
+// ms with the late hits of one step of a warp together, -> 0.52 ms gathered over
+// its steps).  REF: the reference formula's order of operations for the points
+// (the FP64 re-render), else the render's.  its: DQ iterations, on six-lane
+// groups' first lanes.
+template <int SQ, int MOD, bool REF>
+__device__ __forceinline__ void late_normals(const FrameDesc &fd, const int4 *list, int count, unsigned long long &its)
 {
     const FrameT<double> &F = fd.d;
     const int lane = threadIdx.x & 31;
-    do {
-        const int x = pixel % fd.W, y = pixel / fd.W;
-        npx += lane == 0 ? 1 : 0;
-        double d[3], t_in, t_out;
-        if (!camera_clip<double>(F, fd.W, fd.H, x, y, d, t_in, t_out)) {
-            if (lane == 0) write_miss<double>(fd, x, y, 0);
-            break;
-        }
+    const int grp = lane / 6, q = lane - 6 * grp;  // lanes 30 and 31 idle
+    const bool part = grp < count && grp < kLateGroup;
+    int4 e = list[part ? grp : 0];
+    const int ns = part ? e.y : 0;
+    const int nmax = __reduce_max_sync(kFull, ns);
+    const int x = e.x & 0xffff, y = e.x >> 16;
+    const double t = __longlong_as_double(((long long)e.w << 32) | (long long)(unsigned)e.z);
+    double d[3], t_in, t_out, z[8];
+    camera_clip<double>(F, fd.W, fd.H, x, y, d, t_in, t_out);
+    const int a = q >> 1;
+    const double hs = (q & 1) == 0 ? F.h : -F.h;
+    if (REF) {
+        double p[3] = {F.eye[0] + t * d[0], F.eye[1] + t * d[1], F.eye[2] + t * d[2]};
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            if (i == a) p[i] += hs;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) z[j] = F.O[j] + p[0] * F.E[0][j] + p[1] * F.E[1][j] + p[2] * F.E[2][j];
+    } else {
+        double D[8];
+        slice_dir<double>(F, d, D);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) z[i] = fma(hs, F.E[a][i], fma(t, D[i], F.A[i]));
+    }
+    double sp = dq_sp<double>(z);
+#pragma unroll 1
+    for (int n = 0; n < nmax; ++n)
+        if (n < ns) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
+    const double fv = modulus<double, MOD>(z);
+    const unsigned bad = __ballot_sync(kFull, !(fv <= normal_fmax(0.0)));
+    double f[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) f[i] = __shfl_sync(kFull, fv, min(6 * grp, 24) + i);
+    if (part && q == 0) {
+        const double g[3] = {f[0] - f[1], f[2] - f[3], f[4] - f[5]};
+        its += 6ull * (unsigned)ns;
+        shade_write<double>(fd, F, x, y, ns, t, g, ((bad >> (6 * grp)) & 63u) != 0, d);
+    }
+    __syncwarp();
+}
+
+// Add the lanes' late hits to the warp's list (room for kLateGroup - 1 + 32) and
+// evaluate full groups; n: entries in the list (warp-uniform).
+template <int SQ, int MOD>
+__device__ __forceinline__ void push_late(const FrameDesc &fd, bool flag, int4 hit, int4 *list, int &n,
+                                          unsigned long long &its)
+{
+    const unsigned m = __ballot_sync(kFull, flag);
+    if (m == 0) return;
+    if (flag) list[n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u))] = hit;
+    n += __popc(m);
+    __syncwarp();
+#pragma unroll 1
+    while (n >= kLateGroup) {
+        n -= kLateGroup;
+        late_normals<SQ, MOD, false>(fd, list + n, kLateGroup, its);
+    }
+}
+
+// Re-render of the pixels dirty_list[first, first + count), count <= 5, by one
+// warp (all 32 lanes call), with the oracle's formulas for the sample positions
+// (the reference sequence of steps) in FP64; a march or bisection sample is
+// classified in FP32 where the rounding bound decides (count_bound), else by
+// count64.  The pixels' camera rays are set up on one lane each, their samples
+// are taken pixel by pixel: the lanes classify 32 consecutive march samples at
+// a time, a ballot finds the first inside one and warp reductions give the
+// largest escape count before it, so the result and the iteration count are
+// those of the sample-by-sample loop; the bisection runs five levels per round
+// across the lanes.  The hits' FP64 normals are evaluated together at the end
+// (list: room for five entries).  A warp instruction in FP64 takes the same time
+// for one lane as for 32: one pixel at a time the ray setup and the normal took
+// most of the pass (1080p, default c, 9,940 pixels: 0.57 -> 0.36 ms).  Adds the
+// iterations to its (per lane) and the pixels to npx (lane 0).
+template <int SQ, int MOD>
+__device__ __forceinline__ void fixup_pixels(const FrameDesc &fd, const Scratch &sc, unsigned first, int count,
+                                             TileBox &box, int4 *list, unsigned long long &its,
+                                             unsigned long long &npx)
+{
+    const FrameT<double> &F = fd.d;
+    const int lane = threadIdx.x & 31;
+    npx += lane == 0 ? (unsigned)count : 0;
+    int px = 0, py = 0, hits = 0;
+    double pd[3], p_in, p_out;
+    {
+        const int pixel = lane < count ? __ldcg(sc.dirty_list + first + lane) : 0;
+        px = pixel % fd.W;
+        py = pixel / fd.W;
+    }
+    const bool crosses = camera_clip<double>(F, fd.W, fd.H, px, py, pd, p_in, p_out);
+    if (lane < count && !crosses) write_miss<double>(fd, px, py, 0);
+    unsigned todo = __ballot_sync(kFull, lane < count && crosses);
+#pragma unroll 1
+    while (todo) {
+        const int who = __ffs(todo) - 1;
+        todo &= todo - 1;
+        const int x = __shfl_sync(kFull, px, who), y = __shfl_sync(kFull, py, who);
+        const double d[3] = {__shfl_sync(kFull, pd[0], who), __shfl_sync(kFull, pd[1], who),
+                             __shfl_sync(kFull, pd[2], who)};
+        const double t_in = __shfl_sync(kFull, p_in, who), t_out = __shfl_sync(kFull, p_out, who);
         const double delta = (t_out - t_in) / (double)fd.N;
         auto slice = [&](double t, double (&z)[8]) {
             auto comp = [&](int j) {
@@ -716,7 +814,7 @@ __device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, Tile
         }
         if (k_first < 0) {
             if (lane == 0) write_miss<double>(fd, x, y, esc_max);
-            break;
+            continue;
         }
         double depth = t_in;
         int n_star = fd.max_iter;
@@ -762,27 +860,11 @@ __device__ __forceinline__ void fixup_pixel(const FrameDesc &fd, int pixel, Tile
             }
             depth = lo + 0.5 * (hi - lo);
         }
-        // normal: lane 2a + s evaluates F at p +- h e_a
-        double fv = 0.0;
-        if (lane < 6) {
-            const int a = lane >> 1;
-            double p[3] = {F.eye[0] + depth * d[0], F.eye[1] + depth * d[1], F.eye[2] + depth * d[2]};
-            p[a] += (lane & 1) == 0 ? F.h : -F.h;
-            double z[8];
-            for (int j = 0; j < 8; ++j) z[j] = F.O[j] + p[0] * F.E[0][j] + p[1] * F.E[1][j] + p[2] * F.E[2][j];
-            double sp = dq_sp<double>(z);
-#pragma unroll 1
-            for (int n = 0; n < n_star; ++n) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
-            its += (unsigned)n_star;
-            fv = modulus<double, MOD>(z);
-        }
-        const bool bad = lane < 6 && !(fv <= normal_fmax(0.0));
-        const bool guard = __any_sync(kFull, bad);
-        double g[3];
-#pragma unroll
-        for (int a = 0; a < 3; ++a) g[a] = __shfl_sync(kFull, fv, 2 * a) - __shfl_sync(kFull, fv, 2 * a + 1);
-        if (lane == 0) shade_write<double>(fd, F, x, y, n_star, depth, g, guard, d);
-    } while (false);
+        if (lane == 0) list[hits] = late_hit(x, y, n_star, depth);
+        ++hits;
+    }
+    __syncwarp();
+    if (hits) late_normals<SQ, MOD, true>(fd, list, hits, its);
 }
 
 // Device clock in nanoseconds, for the time limits of bounded waits.
@@ -1369,64 +1451,13 @@ __device__ __forceinline__ void normal_shade(const FrameDesc &fd, const FrameT<T
     }
 }
 
-// FP64 normals and shading of the hits of the lanes in `mask` (pixel (x, y),
-// depth and n* on those lanes; all 32 lanes call): five hits at a time, the six
-// field evaluations of a hit on six lanes, on the hit's FP64 ray.  The normals
-// of a recheck frame with more than late_step steps come here.  An FP64 warp
-// instruction takes the same time for one lane as for 32, so evaluating the six
-// in turn on the hits' own lanes, or on the four lanes of a hit's group, wasted
-// the lanes of the other hits (512 x 512, max_iter 24, 55 % of the hits late:
-// bisection pass 0.74 -> 0.63 ms).
-template <int SQ, int MOD>
-__device__ __forceinline__ void late_normals(const FrameDesc &fd, unsigned mask, int x, int y, double depth, int n_star,
-                                             LaneStats &st)
-{
-    const FrameT<double> &F = fd.d;
-    const int lane = threadIdx.x & 31;
-    const int grp = lane / 6, q = lane - 6 * grp;  // lanes 30 and 31 idle
-    while (mask) {
-        int src = -1, nmax = 0;
-#pragma unroll
-        for (int j = 0; j < 5; ++j) {
-            const int b = mask ? __ffs(mask) - 1 : -1;
-            mask &= mask - 1;
-            if (grp == j) src = b;
-            if (b >= 0) nmax = max(nmax, __shfl_sync(kFull, n_star, b));
-        }
-        const int from = src < 0 ? 0 : src;
-        const int hx = __shfl_sync(kFull, x, from), hy = __shfl_sync(kFull, y, from);
-        const int ns = __shfl_sync(kFull, n_star, from);
-        const double t = __shfl_sync(kFull, depth, from);
-        double d[3], D[8], t_in, t_out;
-        camera_clip<double>(F, fd.W, fd.H, hx, hy, d, t_in, t_out);
-        slice_dir<double>(F, d, D);
-        const int a = q >> 1;
-        const double hs = (q & 1) == 0 ? F.h : -F.h;
-        double z[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) z[i] = fma(hs, F.E[a][i], fma(t, D[i], F.A[i]));
-        double sp = dq_sp<double>(z);
-#pragma unroll 1
-        for (int n = 0; n < nmax; ++n)
-            if (n < ns) dq_iter<double, SQ, MOD>(z, z, sp, F.c);
-        const double fv = modulus<double, MOD>(z);
-        const unsigned bad = __ballot_sync(kFull, !(fv <= normal_fmax(0.0)));
-        double f[6];
-#pragma unroll
-        for (int i = 0; i < 6; ++i) f[i] = __shfl_sync(kFull, fv, min(6 * grp, 24) + i);
-        if (src >= 0 && q == 0) {
-            const double g[3] = {f[0] - f[1], f[2] - f[3], f[4] - f[5]};
-            st.niters += 6ull * (unsigned)ns;
-            shade_write<double>(fd, F, hx, hy, ns, t, g, ((bad >> (6 * grp)) & 63u) != 0, d);
-        }
-    }
-}
-
 // Bisection, normal and shading of hit-list entries [base, base + 32) clipped to
-// nhits, one per lane (see bisect_kernel); all 32 lanes call.
+// nhits, one per lane (see bisect_kernel); all 32 lanes call.  Late hits of the
+// recheck mode join the warp's list late[0, nlate) (push_late); the caller
+// evaluates what is left in it.
 template <typename T, int SQ, int MOD, bool RECHECK>
 __device__ __forceinline__ void bisect_chunk(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nhits,
-                                             LaneStats &st)
+                                             LaneStats &st, int4 *late, int &nlate)
 {
     const FrameT<T> &F = frame<T>(fd);
     const int lane = threadIdx.x & 31;
@@ -1508,7 +1539,7 @@ __device__ __forceinline__ void bisect_chunk(const FrameDesc &fd, const Scratch 
     const bool n64 = RECHECK && sizeof(T) == 4 && part && n_lo > late_step<MOD>();
     normal_shade<T, SQ, MOD>(fd, F, x, y, d, D, depth, n_lo, part && !n64, st);
     if constexpr (RECHECK && sizeof(T) == 4)
-        late_normals<SQ, MOD>(fd, __ballot_sync(kFull, n64), x, y, (double)depth, n_lo, st);
+        push_late<SQ, MOD>(fd, n64, late_hit(x, y, n_lo, (double)depth), late, nlate, st.niters);
     st.iters += iters;
     st.samples += samples;
 }
@@ -1569,7 +1600,7 @@ __device__ __forceinline__ void group_normal(const FrameDesc &fd, const FrameT<U
 // those of bisect_chunk.
 template <typename T, int SQ, int MOD, bool RECHECK, int L>
 __device__ __forceinline__ void bisect_group(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nhits,
-                                             LaneStats &st)
+                                             LaneStats &st, int4 *late, int &nlate)
 {
     static_assert(L == 4 || L == 8, "four or eight lanes per hit");
     constexpr int kLevels = L == 8 ? 3 : 2;  // tree levels per round
@@ -1672,7 +1703,7 @@ __device__ __forceinline__ void bisect_group(const FrameDesc &fd, const Scratch 
     const bool n64 = RECHECK && sizeof(T) == 4 && part && n_lo > late_step<MOD>();
     group_normal<T, SQ, MOD, L>(fd, F, x, y, d, D, depth, n_lo, part && !n64, st);
     if constexpr (RECHECK && sizeof(T) == 4)
-        late_normals<SQ, MOD>(fd, __ballot_sync(kFull, n64 && j == 0), x, y, (double)depth, n_lo, st);
+        push_late<SQ, MOD>(fd, n64 && j == 0, late_hit(x, y, n_lo, (double)depth), late, nlate, st.niters);
     if (part && j == 0) {
         st.iters += iters;
         st.samples += samples;

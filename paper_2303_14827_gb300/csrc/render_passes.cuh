@@ -330,6 +330,10 @@ __global__ void __launch_bounds__(kBlock) bisect_kernel(const __grid_constant__ 
     const int lane = threadIdx.x & 31;
     const unsigned nhits = min(*(volatile unsigned *)&sc.ctr->hit_count, sc.hit_cap);
     const int lanes = nhits < group_below ? group_lanes : 1;
+    constexpr bool kLate = RECHECK && sizeof(T) == 4;
+    __shared__ int4 s_late[kLate ? kBlock / 32 : 1][kLate ? kLateGroup + 32 : 1];  // late hits, per warp
+    int4 *late = s_late[kLate ? threadIdx.x >> 5 : 0];
+    int nlate = 0;
     const unsigned per = 32u / (unsigned)lanes;
     LaneStats st;
     for (;;) {
@@ -338,10 +342,12 @@ __global__ void __launch_bounds__(kBlock) bisect_kernel(const __grid_constant__ 
         base = __shfl_sync(kFull, base, 0);
         if (base >= nhits) break;
         if (lanes == 4)
-            bisect_group<T, SQ, MOD, RECHECK, 4>(fd, sc, base, nhits, st);
+            bisect_group<T, SQ, MOD, RECHECK, 4>(fd, sc, base, nhits, st, late, nlate);
         else
-            bisect_chunk<T, SQ, MOD, RECHECK>(fd, sc, base, nhits, st);
+            bisect_chunk<T, SQ, MOD, RECHECK>(fd, sc, base, nhits, st, late, nlate);
     }
+    if constexpr (kLate)
+        if (nlate > 0) late_normals<SQ, MOD, false>(fd, late, nlate, st.niters);
     flush_lane_stats<RECHECK>(sc, st, false);
 }
 
@@ -369,19 +375,21 @@ __global__ void __launch_bounds__(kBlock) recheck_kernel(const __grid_constant__
     // a full queue: pixels whose samples did not fit were flagged by the pushers
 }
 
-// FP64 re-render of the pixels queued by the recheck, one pixel per warp
-// (fixup_pixel).  Pixels go to warps of different blocks first, so a short
-// list spreads over the SMs.
+// FP64 re-render of the pixels queued by the recheck (fixup_pixels), up to five
+// per warp at a time, one while there are fewer pixels than warps.  Pixels go to
+// warps of different blocks first, so a short list spreads over the SMs.
 template <int SQ, int MOD>
 __global__ void __launch_bounds__(kBlock) fixup_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
 {
-    const int lane = threadIdx.x & 31;
-    const unsigned nd = min(*(volatile unsigned *)&sc.ctr->dirty_count, sc.dirty_cap);
-    const unsigned warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, nwarps = gridDim.x * (blockDim.x >> 5);
-    unsigned long long its = 0, npx = 0;
     __shared__ TileBox box[kBlock / 32];
-    for (unsigned i = warp; i < nd; i += nwarps)
-        fixup_pixel<SQ, MOD>(fd, sc.dirty_list[i], box[threadIdx.x >> 5], its, npx);
+    __shared__ int4 list[kBlock / 32][kLateGroup];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned nd = min(*(volatile unsigned *)&sc.ctr->dirty_count, sc.dirty_cap);
+    const unsigned warp = wib * gridDim.x + blockIdx.x, nwarps = gridDim.x * (blockDim.x >> 5);
+    const unsigned per = min((unsigned)kLateGroup, max(1u, (nd + nwarps - 1u) / nwarps));
+    unsigned long long its = 0, npx = 0;
+    for (unsigned i = warp * per; i < nd; i += nwarps * per)
+        fixup_pixels<SQ, MOD>(fd, sc, i, (int)min(per, nd - i), box[wib], list[wib], its, npx);
     const unsigned long long v = warp_sum(its), p = warp_sum(npx);
     if (lane == 0) {
         if (v) atomicAdd(&sc.ctr->stats[6], v);

@@ -12,7 +12,7 @@
 //                  with the FP64 recheck of its staged samples);
 //   BISECT phase : 32 hit-list entries (bisect_chunk);
 //   RECHECK phase: 32 recheck-queue entries (recheck_entry), recheck mode only;
-//   FIXUP phase  : one pixel to re-render in FP64 (fixup_pixel), recheck mode.
+//   FIXUP phase  : one to five pixels to re-render in FP64 (fixup_pixels), recheck mode.
 // The warp that completes a phase's last item moves the request to the next
 // phase that has work.  The warp that completes its last item copies the
 // request's counters to the caller's stats array and writes the request's
@@ -180,10 +180,12 @@ __device__ __forceinline__ void march_item(const FrameDesc &fd, const Scratch &s
 }
 
 template <bool RECHECK>
-__device__ __noinline__ void bisect_item(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nh)
+__device__ __noinline__ void bisect_item(const FrameDesc &fd, const Scratch &sc, unsigned base, unsigned nh, int4 *late)
 {
     LaneStats st;
-    bisect_chunk<float, 0, 0, RECHECK>(fd, sc, base, nh, st);
+    int nlate = 0;
+    bisect_chunk<float, 0, 0, RECHECK>(fd, sc, base, nh, st, late, nlate);
+    if (RECHECK && nlate > 0) late_normals<0, 0, false>(fd, late, nlate, st.niters);
     flush_lane_stats<RECHECK>(sc, st, false);
 }
 
@@ -194,13 +196,18 @@ __device__ __noinline__ void recheck_item(const FrameDesc &fd, const Scratch &sc
     __syncwarp();
 }
 
-__device__ __noinline__ void fixup_item(const FrameDesc &fd, const Scratch &sc, unsigned i, TileBox &box)
+__device__ __noinline__ void fixup_item(const FrameDesc &fd, const Scratch &sc, unsigned i, int count, TileBox &box,
+                                        int4 *list)
 {
     unsigned long long its = 0, npx = 0;
-    fixup_pixel<0, 0>(fd, __ldcg(sc.dirty_list + i), box, its, npx);
+    fixup_pixels<0, 0>(fd, sc, i, count, box, list, its, npx);
     flush_stat(&sc.ctr->stats[6], its);
     flush_stat(&sc.ctr->stats[5], npx);
 }
+
+// Pixels of a FIXUP item: five where a request has many, else one, so that a
+// short list spreads over the warps.
+__device__ __forceinline__ unsigned fixup_step(unsigned total) { return total >= 2048u ? (unsigned)kLateGroup : 1u; }
 
 // Claim up to `step` items of a phase (lane 0): the first claimed index, or
 // ~0u when the phase has none left.
@@ -264,7 +271,8 @@ __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
             } else if (ph == kPhaseRecheck) {
                 item = claim(&b->q_claim, ld_vol32(&b->q_total), 32);
             } else if (ph == kPhaseFixup) {
-                item = claim(&b->f_claim, ld_vol32(&b->f_total), 1);
+                const unsigned nf = ld_vol32(&b->f_total);
+                item = claim(&b->f_claim, nf, fixup_step(nf));
             }
         }
         item = __shfl_sync(kFull, item, 0);
@@ -313,9 +321,9 @@ __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
         } else if (ph == kPhaseBisect) {
             const unsigned nh = ld_vol32(&b->hit_total);
             if (recheck)
-                bisect_item<true>(fd, sc, item, nh);
+                bisect_item<true>(fd, sc, item, nh, s_stage[wib]);
             else
-                bisect_item<false>(fd, sc, item, nh);
+                bisect_item<false>(fd, sc, item, nh, nullptr);
             done_ctr = &b->hit_done;
             n_items = min(32u, nh - item);
             total = nh;
@@ -326,10 +334,10 @@ __global__ void __launch_bounds__(kBlock, 3) serve_kernel(ServeCtl ctl)
             n_items = min(32u, nq - item);
             total = nq;
         } else {
-            fixup_item(fd, sc, item, s_box[wib]);
-            done_ctr = &b->f_done;
-            n_items = 1;
             total = ld_vol32(&b->f_total);
+            n_items = min(fixup_step(total), total - item);
+            fixup_item(fd, sc, item, (int)n_items, s_box[wib], s_stage[wib]);
+            done_ctr = &b->f_done;
         }
         __threadfence();
         unsigned long long done = 0;
