@@ -397,7 +397,10 @@ dqj_status dqj_voxelize(dqj_ctx *ctx, const dqj_params *p, int32_t grid_n, uint8
  * occupancy is grid_n^3 bytes of device memory, nonzero = occupied, linear index
  * (k grid_n + j) grid_n + i as written by dqj_voxelize.  The Julia, march and
  * precision fields of p are validated but unused.  Stream-ordered on
- * cuda_stream; uses no context memory.  A choice between two cell faces that
+ * cuda_stream.  Occupancies of blocks of cells (at most 2 MiB) live for the call
+ * in a pool of the context that keeps its memory until dqj_destroy, so calls on
+ * several streams share nothing; under stream capture none is allocated and the
+ * walk goes cell by cell (the same image).  A choice between two cell faces that
  * lie within rounding of each other may go either way.  Errors: DQJ_ERR_INVALID
  * for a bad p or outputs, grid_n outside 1..DQJ_VOXEL_MAX_GRID, NULL occupancy
  * or a mock context; DQJ_ERR_CUDA for a failed launch.

@@ -93,6 +93,7 @@ struct dqj_ctx {
     // dqj_voxelize scratch: counter block + FP64 recheck queue; grow-only
     void *vox_scratch = nullptr;
     size_t vox_bytes = 0;
+    cudaMemPool_t mip_pool = nullptr;  // dqj_render_voxels: block occupancies, one per call in flight
     // profiling ring: ring_frames x 5 events, next slot, renders recorded
     std::vector<cudaEvent_t> ev;
     int ring_frames = 0;

@@ -917,6 +917,7 @@ dqj_status dqj_destroy(dqj_ctx *ctx)
                 if (ctx->host_copied[b]) cudaEventDestroy(ctx->host_copied[b]);
             }
             if (ctx->vox_scratch) cudaFree(ctx->vox_scratch);
+            if (ctx->mip_pool) cudaMemPoolDestroy(ctx->mip_pool);
             if (ctx->host_stream) cudaStreamDestroy(ctx->host_stream);
             if (ctx->host_copy_stream) cudaStreamDestroy(ctx->host_copy_stream);
             if (ctx->done_ev) cudaEventDestroy(ctx->done_ev);
