@@ -160,6 +160,15 @@ __device__ __forceinline__ void flush_stat(unsigned long long *dst, unsigned lon
     if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
 }
 
+// flush_stat of a count below 2^51: two warp reductions of 32-bit parts (24 low
+// bits, and the rest) instead of ten 64-bit shuffles and additions.
+__device__ __forceinline__ void flush_count(unsigned long long *dst, unsigned long long v)
+{
+    const unsigned lo = __reduce_add_sync(kFull, (unsigned)v & 0xffffffu);
+    const unsigned hi = __reduce_add_sync(kFull, (unsigned)(v >> 24));
+    if ((threadIdx.x & 31) == 0 && (lo | hi)) atomicAdd(dst, ((unsigned long long)hi << 24) + lo);
+}
+
 template <typename T>
 __device__ __forceinline__ void write_miss(const FrameDesc &fd, int x, int y, int iter)
 {
@@ -1715,12 +1724,12 @@ __device__ __forceinline__ void bisect_group(const FrameDesc &fd, const Scratch 
 template <bool RECHECK>
 __device__ __forceinline__ void flush_lane_stats(const Scratch &sc, const LaneStats &st, bool march)
 {
-    flush_stat(&sc.ctr->stats[0], st.iters);
-    if (march) flush_stat(&sc.ctr->stats[8], st.iters);
-    flush_stat(&sc.ctr->stats[1], st.niters);
-    flush_stat(&sc.ctr->stats[2], st.samples);
-    flush_stat(&sc.ctr->stats[3], st.hits);
-    if (RECHECK) flush_stat(&sc.ctr->stats[4], st.rechecks);
+    flush_count(&sc.ctr->stats[0], st.iters);
+    if (march) flush_count(&sc.ctr->stats[8], st.iters);
+    if (!march) flush_count(&sc.ctr->stats[1], st.niters);  // a march evaluates no normals
+    flush_count(&sc.ctr->stats[2], st.samples);
+    flush_count(&sc.ctr->stats[3], st.hits);
+    if (RECHECK) flush_count(&sc.ctr->stats[4], st.rechecks);
 }
 
 }  // namespace dqj
