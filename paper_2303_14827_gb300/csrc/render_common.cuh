@@ -888,9 +888,9 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
 // tile the warp drops those whose FP32 count a rounding bound proves
 // (recheck_staged); the others go to the frame's queue for the recheck pass, in
 // blocks of 32 (one atomic).  A tile that fills the stage (kQStage entries per
-// warp; a round adds at most 64) appends the staged entries to the queue as
+// warp; a round adds at most 128) appends the staged entries to the queue as
 // they are.
-constexpr int kQStage = 256;
+constexpr int kQStage = 320;
 // Ray parameter of a half without a sample in the recheck march: its first
 // iterate overflows (modulus +inf) and the later ones are infinite or NaN, so
 // its distance from R^2 never falls within a recheck band.
@@ -1270,6 +1270,11 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
     const bool boxa = acta, boxb = actb;
     int suma = 0, sumb = 0, maxa = 0, maxb = 0, kfa = -1, kfb = -1;
     int qn = RECHECK ? *left : 0, counted = qn;  // staged recheck entries (warp-uniform); left: of earlier tiles
+    if (RECHECK) {
+        __syncwarp();
+        if (lane == 0) box.staged = qn;
+        __syncwarp();
+    }
     const int k0 = SPLIT ? kb : 0, k1 = SPLIT ? ke : N + 1;
     const float2 far = make_float2(kFarT, kFarT);
     bool more = __any_sync(kFull, acta || actb);
@@ -1334,33 +1339,27 @@ __device__ __forceinline__ void march4_tile(const FrameDesc &fd, const PairConst
                                                      cb2, dm, dm2, live);
         }
         if (RECHECK && __any_sync(kFull, fminf(fminf(dm.x, dm.y), fminf(dm2.x, dm2.y)) <= P.margin_t)) {
-            // marginal samples in this round (rare): stage sample k's, then sample k + 1's
-            const unsigned below = (1u << lane) - 1u;
-            {
-                const bool pa = acta && dm.x <= P.margin_t, pb = actb && dm.y <= P.margin_t;
-                const unsigned ba = __ballot_sync(kFull, pa), bb = __ballot_sync(kFull, pb);
-                const int nqa = __popc(ba);
-                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k | (kMarchSample << 16), xya, ina ? 0 : ca + 1);
-                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k | (kMarchSample << 16), xyb, inb ? 0 : cb + 1);
-                qn += nqa + __popc(bb);
-                if (qn > kQStage - 64) {
-                    flush_staged(fd, sc, qs, qn, counted);
-                    qn = counted = 0;
-                }
+            // marginal samples in this round: staged by the lanes that hold them (a
+            // few), through the warp's shared counter
+            const bool pa = acta && dm.x <= P.margin_t, pb = actb && dm.y <= P.margin_t;
+            const bool pa2 = acta && has2 && !ina && dm2.x <= P.margin_t;
+            const bool pb2 = actb && has2 && !inb && dm2.y <= P.margin_t;
+            const int np = (pa ? 1 : 0) + (pb ? 1 : 0) + (pa2 ? 1 : 0) + (pb2 ? 1 : 0);
+            if (np) {
+                int at = atomicAdd(&box.staged, np);
+                const int kk = k | (kMarchSample << 16);
+                if (pa) qs[at++] = make_int4(pixa, kk, xya, ina ? 0 : ca + 1);
+                if (pb) qs[at++] = make_int4(pixb, kk, xyb, inb ? 0 : cb + 1);
+                if (pa2) qs[at++] = make_int4(pixa, kk + 1, xya, ina2 ? 0 : ca2 + 1);
+                if (pb2) qs[at++] = make_int4(pixb, kk + 1, xyb, inb2 ? 0 : cb2 + 1);
             }
-            {
-                const bool pa = acta && has2 && !ina && dm2.x <= P.margin_t;
-                const bool pb = actb && has2 && !inb && dm2.y <= P.margin_t;
-                const unsigned ba = __ballot_sync(kFull, pa), bb = __ballot_sync(kFull, pb);
-                const int nqa = __popc(ba);
-                const int k2 = k + 1;
-                if (pa) qs[qn + __popc(ba & below)] = make_int4(pixa, k2 | (kMarchSample << 16), xya, ina2 ? 0 : ca2 + 1);
-                if (pb) qs[qn + nqa + __popc(bb & below)] = make_int4(pixb, k2 | (kMarchSample << 16), xyb, inb2 ? 0 : cb2 + 1);
-                qn += nqa + __popc(bb);
-                if (qn > kQStage - 64) {
-                    flush_staged(fd, sc, qs, qn, counted);
-                    qn = counted = 0;
-                }
+            __syncwarp();
+            qn = *(volatile int *)&box.staged;
+            if (qn > kQStage - 128) {
+                flush_staged(fd, sc, qs, qn, counted);
+                if (lane == 0) box.staged = 0;
+                __syncwarp();
+                qn = counted = 0;
             }
         }
         // sample k + 1 counts only after an outside sample k (ca2 = 0 without a sample)

@@ -40,6 +40,7 @@ static_assert(kSettleCap < 12 && kSettleCap <= 15, "a settled count is no late s
 struct TileBox {
     float c0[3], dc[3], h0[3], dh[3];
     float rho, e1;  // bounds of the rounding of a sample's position and of its first iterate
+    int staged;     // recheck entries the warp has staged (march4_tile; not part of the box)
 };
 
 __device__ __forceinline__ float warp_min(float v)
@@ -107,7 +108,17 @@ __device__ __forceinline__ void tile_box(const FrameDesc &fd, bool acta, const f
     B.rho = 4e-6f * r;
     B.e1 = 8e-6f * r * r;
     __syncwarp();  // the warp's readers of its previous tile's box are done
-    if ((threadIdx.x & 31) == 0) box = B;
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            box.c0[a] = B.c0[a];
+            box.dc[a] = B.dc[a];
+            box.h0[a] = B.h0[a];
+            box.dh[a] = B.dh[a];
+        }
+        box.rho = B.rho;
+        box.e1 = B.e1;
+    }
     __syncwarp();
 }
 
