@@ -23,6 +23,8 @@ namespace dqj {
 namespace {
 
 constexpr int kDeTileW = 8, kDeTileH = 4;
+constexpr int kDeClasses = 4, kDeFixBlock = 128;
+constexpr unsigned kDeLong = 1024;  // see de_mark
 
 // Lockstep classification with the squared derivative: returns the escape
 // count (0 = inside) and, for an escaped sample, the distance estimate.  AXIS:
@@ -48,22 +50,22 @@ __device__ __forceinline__ int classify_de(T (&z)[8], const FrameT<T> &F, int ma
     // the first step, peeled so that it can take the axis form
     m = AXIS ? dq_iter_axis_first<T, MOD>(z, z, sp, F.c) : dq_iter<T, SQ, MOD>(z, z, sp, F.c);
     if (alive) dm = fmin(dm, fabs(m - F.R2));
-    if (alive && !(m <= F.R2)) {
+    if (alive && !bounded(m, F.R2)) {
         m_esc = m;
         dr2_esc = dr2;
     }
-    alive = alive && (m <= F.R2);
+    alive = alive && bounded(m, F.R2);
     cnt += alive ? 1 : 0;
     if (__any_sync(kFull, alive)) {
         for (int n = 1; n < max_iter; ++n) {
             dr2 = T(4) * m * dr2;
             m = dq_iter<T, SQ, MOD>(z, z, sp, F.c);
             if (alive) dm = fmin(dm, fabs(m - F.R2));
-            if (alive && !(m <= F.R2)) {
+            if (alive && !bounded(m, F.R2)) {
                 m_esc = m;
                 dr2_esc = dr2;
             }
-            alive = alive && (m <= F.R2);
+            alive = alive && bounded(m, F.R2);
             cnt += alive ? 1 : 0;
             if (!__any_sync(kFull, alive)) break;
         }
@@ -99,6 +101,24 @@ __device__ __forceinline__ int classify_de(T (&z)[8], const FrameT<T> &F, int ma
 constexpr float kDeEpsBand = 0.02f;   // relative to epsilon
 constexpr float kDeExitBand = 1e-5f;  // scene units (relative above 1)
 
+// Queue a pixel for the FP64 re-trace, once per frame.  The re-trace starts the
+// longest rays first (see de_fixup_kernel), so a pixel goes to the list of its
+// ray's cost in FP32, iterations plus three per sample: kDeLong and above, half,
+// a quarter, an eighth of it, and the rest in dirty_list.  A typical hit of a
+// full-HD frame costs 150 to 450, one in a hundred 1000, the longest ray 4000
+// (c = (-0.2,0.6,0.2,0.2 | 0.1,0,0,0.05): re-trace 6.4 ms with kDeLong 1024 or
+// 768, 6.8 with 1536, 7.3 with 2048; a random slice frame 6.7, 7.2 with 768).
+// The hit list, which this mode does not use otherwise, holds the lists of long
+// rays, each with room for every pixel of the frame.
+__device__ __forceinline__ void de_mark(const FrameDesc &fd, const Scratch &sc, int pixel, unsigned cost)
+{
+    if (atomicExch(&sc.dirty_flag[pixel], fd.epoch) == fd.epoch) return;
+    const int cls = cost >= kDeLong ? 0 : cost >= kDeLong / 2 ? 1 : cost >= kDeLong / 4 ? 2 : cost >= kDeLong / 8 ? 3 : 4;
+    const unsigned slot = atomicAdd(cls < kDeClasses ? &sc.ctr->long_count[cls] : &sc.ctr->dirty_count, 1u);
+    int *list = cls < kDeClasses ? reinterpret_cast<int *>(sc.hits) + (size_t)cls * sc.hit_cap : sc.dirty_list;
+    if (slot < sc.dirty_cap) list[slot] = pixel;
+}
+
 template <typename T, int SQ, int MOD, bool AXIS, bool RECHECK>
 __device__ __forceinline__ bool de_trace_lane(const FrameDesc &fd, const Scratch &sc, int x, int y, bool valid,
                                               LaneStats &st, T (&d)[3], T (&D)[8], T &depth, int &n_star,
@@ -130,6 +150,7 @@ __device__ __forceinline__ bool de_trace_lane(const FrameDesc &fd, const Scratch
     n_star = 0;
     bool hit = false;
     const int pixel = y * fd.W + x;
+    const unsigned it0 = (unsigned)st.iters;
     while (__any_sync(kFull, act)) {
         T z[8];
 #pragma unroll
@@ -143,7 +164,7 @@ __device__ __forceinline__ bool de_trace_lane(const FrameDesc &fd, const Scratch
             if (warp_push(push, make_int4(pixel, steps, __float_as_int((float)t), n | (stop ? 1 << 16 : 0)), sc.queue,
                           sc.queue_cap, &sc.ctr->queue_count)) {
                 atomicAdd(&sc.ctr->stats[7], 1ull);
-                mark_dirty(fd, sc, pixel);
+                de_mark(fd, sc, pixel, kDeLong);
             }
             st.rechecks += push ? 1 : 0;
         }
@@ -159,13 +180,13 @@ __device__ __forceinline__ bool de_trace_lane(const FrameDesc &fd, const Scratch
             } else {
                 t = t + F.de_scale * dist;
                 act = steps < fd.de_max_steps && t <= t1;
-                if (RECHECK && fabs(t - t1) <= T(kDeExitBand) * max(T(1), fabs(t1))) mark_dirty(fd, sc, pixel);
+                if (RECHECK && fabs(t - t1) <= T(kDeExitBand) * max(T(1), fabs(t1))) de_mark(fd, sc, pixel, kDeLong);
             }
         }
     }
     st.samples += (unsigned)steps;
     st.hits += hit ? 1 : 0;
-    if (RECHECK && hit) mark_dirty(fd, sc, pixel);
+    if (RECHECK && hit) de_mark(fd, sc, pixel, (unsigned)st.iters - it0 + 3u * (unsigned)steps);
     return hit;
 }
 
@@ -232,24 +253,53 @@ __global__ void __launch_bounds__(kBlock) de_recheck_kernel(const __grid_constan
         const bool stop = n == 0 || dist < F.de_eps;
         const bool differs = n != (e.w & 0xffff) || stop != ((e.w >> 16) != 0);
         const bool close = dm <= 0.1 * F.margin || (n != 0 && fabs(dist - F.de_eps) <= 0.5 * kDeEpsBand * F.de_eps);
-        if (differs || close) mark_dirty(fd, sc, pixel);
+        if (differs || close) de_mark(fd, sc, pixel, kDeLong);  // its length unknown
     }
 }
 
-// FP64 re-trace of the pixels queued by the recheck, 32 per warp (one per
-// lane, in lockstep like de_kernel), shaded in place.  AXIS: an axis-aligned
-// slice, whose samples take the axis form of the first step (same results).
+// FP64 re-trace of the queued pixels, 32 per warp (one per lane, in lockstep like
+// de_kernel), shaded in place.  AXIS: an axis-aligned slice, whose samples take
+// the axis form of the first step (same results).
+//
+// Bound by the FP64 pipe, 32 to 38 ns per warp instruction and SM quarter, and by
+// the longest ray: 4000 iterations one after the other are 4 ms of instructions
+// that share that pipe with whatever else runs on their SM quarter.  So each
+// quarter runs one warp (it alone keeps the pipe busy), and warps claim 32 pixels
+// at a time from the lists in the order of their rays' cost: the long rays start
+// first, run at the pipe's full rate, and the short ones fill the end.  Against
+// strided shares of one list at four blocks per SM: 9.5 -> 6.4 ms at 1920x1080,
+// c = (-0.2,0.6,0.2,0.2 | 0.1,0,0,0.05); 3.6 -> 2.4 and 6.2 -> 3.5 ms at random c,
+// 9.8 -> 6.7 ms on a random slice frame.  Two and three warps per quarter took 6.8
+// and 8.0 ms.  Claims of single pixels by idle lanes (no lockstep) executed 28 %
+// more instructions: neighbours' samples escape at much the same step.
 template <int SQ, int MOD, bool AXIS>
-__global__ void __launch_bounds__(kBlock) de_fixup_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
+__global__ void __launch_bounds__(kDeFixBlock) de_fixup_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
 {
     const FrameT<double> &F = fd.d;
     const int lane = threadIdx.x & 31;
-    const unsigned nd = min(*(volatile unsigned *)&sc.ctr->dirty_count, sc.dirty_cap);
+    // chunks of 32 pixels, the lists one after the other from the longest rays down
+    unsigned end[kDeClasses + 1], chunks = 0;
+#pragma unroll
+    for (int c = 0; c <= kDeClasses; ++c) {
+        const unsigned n = *(volatile unsigned *)(c < kDeClasses ? &sc.ctr->long_count[c] : &sc.ctr->dirty_count);
+        end[c] = chunks += (min(n, sc.dirty_cap) + 31) / 32;
+    }
     const unsigned warp = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, nwarps = gridDim.x * (blockDim.x >> 5);
     LaneStats st, st_fix;
-    for (unsigned base = warp * 32; base < nd; base += nwarps * 32) {
-        const bool valid = base + lane < nd;
-        const int pixel = valid ? sc.dirty_list[base + lane] : 0;
+    for (unsigned chunk = warp; chunk < chunks;) {
+        int c = 0;
+        unsigned first = 0;
+#pragma unroll
+        for (int k = 0; k < kDeClasses; ++k)
+            if (chunk >= end[k]) {
+                c = k + 1;
+                first = end[k];
+            }
+        const unsigned i = (chunk - first) * 32 + lane;
+        const unsigned n = c < kDeClasses ? sc.ctr->long_count[c] : sc.ctr->dirty_count;
+        const int *list = c < kDeClasses ? reinterpret_cast<const int *>(sc.hits) + (size_t)c * sc.hit_cap : sc.dirty_list;
+        const bool valid = i < min(n, sc.dirty_cap);
+        const int pixel = valid ? list[i] : 0;
         const int x = pixel % fd.W, y = pixel / fd.W;
         double d[3], D[8], depth;
         int n_star, esc_max;
@@ -258,6 +308,8 @@ __global__ void __launch_bounds__(kBlock) de_fixup_kernel(const __grid_constant_
         if (valid && !hit) write_miss<double>(fd, x, y, esc_max);
         normal_shade<double, SQ, MOD>(fd, F, x, y, d, D, depth, n_star, hit, st_fix);
         st.hits += valid ? 1 : 0;
+        if (lane == 0) chunk = nwarps + atomicAdd(&sc.ctr->dirty_next, 1u);
+        chunk = __shfl_sync(kFull, chunk, 0);
     }
     flush_stat(&sc.ctr->stats[5], st.hits);
     flush_stat(&sc.ctr->stats[6], st_fix.iters + st_fix.niters);
@@ -312,19 +364,17 @@ cudaError_t launch_de_t(const FrameDesc &fd, const Scratch &sc, cudaStream_t st,
     else
         de_kernel<T, SQ, MOD, false, RECHECK><<<gd > 0 ? gd : 1, kBlock, 0, st>>>(fd, sc);
     if (ev) cudaEventRecord(ev[1], st);
-    de_shade_kernel<T, SQ, MOD><<<gs > 0 ? gs : 1, kBlock, 0, st>>>(fd, sc);
+    if constexpr (!RECHECK) de_shade_kernel<T, SQ, MOD><<<gs > 0 ? gs : 1, kBlock, 0, st>>>(fd, sc);
     if (ev) cudaEventRecord(ev[2], st);
     if constexpr (RECHECK) {
-        static std::atomic<int> g_re{0}, g_fx{0}, g_fxg{0};
+        static std::atomic<int> g_re{0};
         de_recheck_kernel<SQ, MOD><<<num_sms * resident_per_sm(g_re, de_recheck_kernel<SQ, MOD>), kBlock, 0, st>>>(
             fd, sc);
         if (ev) cudaEventRecord(ev[3], st);
         if (fd.axis_slice)
-            de_fixup_kernel<SQ, MOD, true>
-                <<<num_sms * resident_per_sm(g_fx, de_fixup_kernel<SQ, MOD, true>), kBlock, 0, st>>>(fd, sc);
+            de_fixup_kernel<SQ, MOD, true><<<num_sms, kDeFixBlock, 0, st>>>(fd, sc);
         else
-            de_fixup_kernel<SQ, MOD, false>
-                <<<num_sms * resident_per_sm(g_fxg, de_fixup_kernel<SQ, MOD, false>), kBlock, 0, st>>>(fd, sc);
+            de_fixup_kernel<SQ, MOD, false><<<num_sms, kDeFixBlock, 0, st>>>(fd, sc);
         if (ev) cudaEventRecord(ev[4], st);
     } else if (ev) {
         cudaEventRecord(ev[3], st);

@@ -49,6 +49,16 @@ __host__ __device__ constexpr int late_step() { return MOD == 1 ? 12 : 20; }
 __device__ __forceinline__ float dfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ double dfma(double a, double b, double c) { return fma(a, b, c); }
 
+// m <= R2 for a modulus m (a sum of squares).  In double on the integer units:
+// non-negative doubles are ordered like their bits, and a NaN of either sign lies
+// above every R2.  An FP64 compare holds the FP64 pipe as long as a
+// multiplication: the re-trace of sphere tracing took 6.8 ms with it, 6.4 so.
+__device__ __forceinline__ bool bounded(float m, float R2) { return m <= R2; }
+__device__ __forceinline__ bool bounded(double m, double R2)
+{
+    return (unsigned long long)__double_as_longlong(m) <= (unsigned long long)__double_as_longlong(R2);
+}
+
 // sp of zeta: r1^2 + r2^2 + r3^2
 template <typename T>
 __device__ __forceinline__ T dq_sp(const T (&z)[8])
@@ -136,12 +146,12 @@ __device__ __forceinline__ int classify_lockstep(T (&z)[8], const FrameT<T> &F, 
     for (int n = 0; n < max_iter; n += 2) {
         T m = dq_iter<T, SQ, MOD>(z, w, sp, F.c);
         if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
-        alive = alive && (m <= F.R2);
+        alive = alive && bounded(m, F.R2);
         cnt += alive ? 1 : 0;
         if (!__any_sync(0xffffffffu, alive) || n + 1 >= max_iter) break;
         m = dq_iter<T, SQ, MOD>(w, z, sp, F.c);
         if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
-        alive = alive && (m <= F.R2);
+        alive = alive && bounded(m, F.R2);
         cnt += alive ? 1 : 0;
         if (!__any_sync(0xffffffffu, alive)) break;
     }
@@ -175,7 +185,7 @@ __device__ __forceinline__ int classify_lockstep_it1(T (&z)[8], const FrameT<T> 
     T sp = dq_sp<T>(z);
     T m = modulus_sp<T, MOD>(z, sp);
     bool mg = RECHECK && alive && fabs(m - F.R2) <= F.margin;
-    alive = alive && (m <= F.R2);
+    alive = alive && bounded(m, F.R2);
     int cnt = alive ? 1 : 0;
     T w[8];
     if (__any_sync(0xffffffffu, alive)) {
@@ -183,12 +193,12 @@ __device__ __forceinline__ int classify_lockstep_it1(T (&z)[8], const FrameT<T> 
         for (int n = 1; n < max_iter; n += 2) {
             m = dq_iter<T, SQ, MOD>(z, w, sp, F.c);
             if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
-            alive = alive && (m <= F.R2);
+            alive = alive && bounded(m, F.R2);
             cnt += alive ? 1 : 0;
             if (!__any_sync(0xffffffffu, alive) || n + 1 >= max_iter) break;
             m = dq_iter<T, SQ, MOD>(w, z, sp, F.c);
             if (RECHECK) mg = mg || (alive && fabs(m - F.R2) <= F.margin);
-            alive = alive && (m <= F.R2);
+            alive = alive && bounded(m, F.R2);
             cnt += alive ? 1 : 0;
             if (!__any_sync(0xffffffffu, alive)) break;
         }

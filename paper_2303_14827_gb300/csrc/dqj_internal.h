@@ -98,14 +98,16 @@ struct Counters {
     unsigned int queue_next;
     unsigned int dirty_count;     // pixels to re-render in FP64
     unsigned int dirty_next;
-    unsigned int pad[5];
+    unsigned int long_count[4];   // sphere tracing: pixels in the lists of long rays (de.cu)
+    unsigned int pad[1];
 };
 static_assert(sizeof(Counters) == 128, "Counters layout");
 
 // Views into one scratch allocation owned by a context.
 struct alignas(16) Scratch {
     Counters *ctr;
-    int4 *hits;           // march: {pixel, k_first, 0, 0}; sphere tracing: {pixel, depth bits, n*}
+    int4 *hits;           // march: {pixel, k_first, 0, 0}; sphere tracing: {pixel, depth bits, n*},
+                          // in its recheck mode the lists of long rays
     uint32_t hit_cap;
     int4 *queue;          // {pixel, k | b << 16, path, n32}
     uint32_t queue_cap;
