@@ -5,7 +5,8 @@
 //             march in step: every trip of the warp classifies sample k of each
 //             lane's ray (Method, "Ray-Marching": fixed steps over the box), so
 //             neighbouring rays - which see almost the same escape counts - share
-//             trips and no lane diverges.  Misses write their final outputs;
+//             trips and no lane diverges.  Runs of samples whose count a bound
+//             proves for the whole tile are not iterated (settle.cuh).  Misses write their final outputs;
 //             hits are appended to a compacted hit list.
 //   bisect  : one hit per lane: B bisection steps of the first outside->inside
 //             bracket, then the six central-difference evaluations of the normal
@@ -14,9 +15,10 @@
 //             near-surface classifications together instead of stalling warps
 //             that are still marching.
 //   recheck : (FP32_RECHECK) samples whose modulus came within the margin of R^2
-//             are re-evaluated in FP64 from FP64 ray parameters, one per thread;
-//             a pixel whose FP64 escape count differs is queued for
-//   fixup   : a complete FP64 re-render of that pixel, one per thread.
+//             and whose count the FP32 orbit's rounding bound leaves open are
+//             decided from FP64 ray parameters, by a two-float orbit and its
+//             bound, else in FP64, gathered; a pixel whose count differs goes to
+//   fixup   : a re-render of that pixel at FP64 accuracy, five pixels per warp.
 // Iteration counts are the algorithmic ones (escape count, or max_iter for an
 // inside sample), accumulated per lane and added once per warp.
 #pragma once
@@ -228,6 +230,15 @@ __global__ void __launch_bounds__(kBlock, AXIS && !(RECHECK && SETTLE) ? 4 : 3) 
     if (RECHECK) flush_rest(fd, sc, qs, left);
 }
 
+// A small frame's three kernels follow one another within 90 us, of which the
+// gaps between them are several (256x256: 88.4 -> 85.3 us).  The two later ones are launched as programmatic
+// dependents (launch_after): they are put on the SMs while the one before still
+// runs, once all its CTAs have started (start_next), and wait for its end and its
+// writes before they read anything (wait_previous).  Neither does anything in a
+// kernel launched the usual way.
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // split march, for frames with fewer tiles than the GPU has resident warps: a
 // work item is one 64-ray tile and one of fd.k_split contiguous ranges of the
@@ -240,6 +251,7 @@ __global__ void __launch_bounds__(kBlock, AXIS && !(RECHECK && SETTLE) ? 4 : 3) 
 template <int SQ, int MOD, bool AXIS>
 __global__ void __launch_bounds__(kBlock, AXIS ? 5 : 4) march2_split_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
 {
+    start_next();
     const int lane = threadIdx.x & 31;
     const unsigned ntiles = subset_tiles(fd, (unsigned)fd.tiles_x * (unsigned)fd.tiles_y);
     const unsigned items = ntiles * (unsigned)fd.k_split;
@@ -262,6 +274,7 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_split_kernel(cons
                                                                             const Scratch sc)
 {
     __shared__ TileBox box[kBlock / 32];
+    start_next();
     const int lane = threadIdx.x & 31;
     const unsigned ntiles = subset_tiles(fd, (unsigned)fd.tiles_x * (unsigned)fd.tiles_y);
     const unsigned items = ntiles * (unsigned)fd.k_split;
@@ -283,6 +296,8 @@ __global__ void __launch_bounds__(kBlock, AXIS ? 4 : 3) march4_split_kernel(cons
 // and samples.
 __global__ void __launch_bounds__(kBlock) march_merge_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc)
 {
+    start_next();
+    wait_previous();
     const int64_t npx = (int64_t)fd.W * fd.H;
     LaneStats st;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < npx; base += (int64_t)gridDim.x * blockDim.x) {
@@ -327,6 +342,7 @@ template <typename T, int SQ, int MOD, bool RECHECK>
 __global__ void __launch_bounds__(kBlock) bisect_kernel(const __grid_constant__ FrameDesc fd, const Scratch sc,
                                                         unsigned group_below, int group_lanes)
 {
+    wait_previous();
     const int lane = threadIdx.x & 31;
     const unsigned nhits = min(*(volatile unsigned *)&sc.ctr->hit_count, sc.hit_cap);
     const int lanes = nhits < group_below ? group_lanes : 1;
@@ -419,6 +435,22 @@ unsigned bisect_group_below(int capb)
     return (unsigned)capb * 4u * 32u;
 }
 
+// Launch on st; `dependent`: as a programmatic dependent of the kernel before it.
+template <typename... P, typename... A>
+void launch_after(bool dependent, void (*kernel)(P...), int grid, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kBlock);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = dependent ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // the error stays for cudaGetLastError
+}
+
 template <int SQ, int MOD, bool RECHECK, bool AXIS, bool SETTLE>
 void launch_march4(const FrameDesc &fd, const Scratch &sc, cudaStream_t st, int num_sms, unsigned ntiles)
 {
@@ -433,9 +465,14 @@ cudaError_t launch_passes(const FrameDesc &fd, const Scratch &sc, cudaStream_t s
 {
     static std::atomic<int> g_march{0}, g_marchg{0}, g_march2a{0}, g_march2g{0}, g_bisect{0};
     const unsigned ntiles = subset_tiles(fd, (unsigned)fd.tiles_x * (unsigned)fd.tiles_y);
+    // split frames: not under capture (a captured graph keeps plain edges), nor
+    // with an event between the kernels
+    bool dependent = false;
     if (ev) cudaEventRecord(ev[0], st);
     if constexpr (sizeof(T) == 4 && !RECHECK) {
         if (fd.march_variant == 1 && fd.k_split > 1) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            dependent = !ev && cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
             static std::atomic<int> g_sa{0}, g_sg{0}, g_mg{0};
             const unsigned items = ntiles * (unsigned)fd.k_split;
             if (fd.march_samples == 2) {
@@ -458,7 +495,7 @@ cudaError_t launch_passes(const FrameDesc &fd, const Scratch &sc, cudaStream_t s
             }
             const unsigned npx = (unsigned)fd.W * (unsigned)fd.H;
             const int capm = num_sms * resident_per_sm(g_mg, march_merge_kernel);
-            march_merge_kernel<<<(int)min((unsigned)capm, (npx + kBlock - 1) / kBlock), kBlock, 0, st>>>(fd, sc);
+            launch_after(dependent, march_merge_kernel, (int)min((unsigned)capm, (npx + kBlock - 1) / kBlock), st, fd, sc);
         }
     }
     if constexpr (sizeof(T) == 4) {
@@ -498,8 +535,8 @@ cudaError_t launch_passes(const FrameDesc &fd, const Scratch &sc, cudaStream_t s
     const int capb = num_sms * resident_per_sm(g_bisect, bisect_kernel<T, SQ, MOD, RECHECK>);
     const unsigned maxw = ((unsigned)fd.W * (unsigned)fd.H + 31u) / 32u;
     const int gb = (int)min((unsigned)capb, (maxw + 3u) / 4u);
-    bisect_kernel<T, SQ, MOD, RECHECK><<<gb > 0 ? gb : 1, kBlock, 0, st>>>(fd, sc, bisect_group_below(capb),
-                                                                          bisect_group_lanes());
+    launch_after(dependent, bisect_kernel<T, SQ, MOD, RECHECK>, gb > 0 ? gb : 1, st, fd, sc, bisect_group_below(capb),
+                 bisect_group_lanes());
     if (ev) cudaEventRecord(ev[2], st);
     if (RECHECK) {
         static std::atomic<int> g_re{0}, g_fx{0};
