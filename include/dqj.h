@@ -51,9 +51,9 @@ typedef enum {
 /* dqj_params.precision */
 enum {
     DQJ_FP32 = 0,         /* FP32 throughout                                         */
-    DQJ_FP32_RECHECK = 1, /* FP32, samples within recheck_margin of R^2 re-evaluated
-                             in FP64 on the GPU; a pixel whose FP64 decision differs
-                             is re-rendered in FP64                                  */
+    DQJ_FP32_RECHECK = 1, /* FP32, samples within recheck_margin of R^2 decided at
+                             FP64 accuracy on the GPU (a rounding bound, or FP64);
+                             a pixel whose decision differs is re-rendered so        */
     DQJ_FP64 = 2          /* FP64 throughout                                         */
 };
 
@@ -179,7 +179,7 @@ enum {
     DQJ_STAT_NORMAL_ITERS = 1, /* DQ iterations of the six normal evaluations         */
     DQJ_STAT_SAMPLES = 2,      /* classified samples (march + bisection, or DE)       */
     DQJ_STAT_HITS = 3,         /* hit pixels                                          */
-    DQJ_STAT_RECHECKS = 4,     /* samples re-evaluated in FP64                        */
+    DQJ_STAT_RECHECKS = 4,     /* samples rechecked: by a rounding bound, or in FP64  */
     DQJ_STAT_FIXUPS = 5,       /* pixels re-rendered in FP64 after a disagreement     */
     DQJ_STAT_FIXUP_ITERS = 6,  /* DQ iterations spent by those re-renders             */
     DQJ_STAT_OVERFLOW = 7,     /* recheck-queue overflows (pixel re-rendered instead) */
