@@ -46,7 +46,7 @@ __device__ __forceinline__ int classify_de(T (&z)[8], const FrameT<T> &F, int ma
         sp = dq_sp<T>(z);
         m = modulus<T, MOD>(z);
     }
-    T dr2 = T(4) * m, m_esc = T(0), dr2_esc = T(1);
+    T dr2 = four_times(m), m_esc = T(0), dr2_esc = T(1);
     // the first step, peeled so that it can take the axis form
     m = AXIS ? dq_iter_axis_first<T, MOD>(z, z, sp, F.c) : dq_iter<T, SQ, MOD>(z, z, sp, F.c);
     if (alive) dm = fmin(dm, fabs(m - F.R2));
@@ -58,7 +58,7 @@ __device__ __forceinline__ int classify_de(T (&z)[8], const FrameT<T> &F, int ma
     cnt += alive ? 1 : 0;
     if (__any_sync(kFull, alive)) {
         for (int n = 1; n < max_iter; ++n) {
-            dr2 = T(4) * m * dr2;
+            dr2 = four_times(m) * dr2;
             m = dq_iter<T, SQ, MOD>(z, z, sp, F.c);
             if (alive) dm = fmin(dm, fabs(m - F.R2));
             if (alive && !bounded(m, F.R2)) {
@@ -267,7 +267,8 @@ __global__ void __launch_bounds__(kBlock) de_recheck_kernel(const __grid_constan
 // quarter runs one warp (it alone keeps the pipe busy), and warps claim 32 pixels
 // at a time from the lists in the order of their rays' cost: the long rays start
 // first, run at the pipe's full rate, and the short ones fill the end.  Against
-// strided shares of one list at four blocks per SM: 9.5 -> 6.4 ms at 1920x1080,
+// strided shares of one list at four blocks per SM: 9.5 -> 6.4 ms (6.0 with the
+// integer doubling of dq_math.cuh) at 1920x1080,
 // c = (-0.2,0.6,0.2,0.2 | 0.1,0,0,0.05); 3.6 -> 2.4 and 6.2 -> 3.5 ms at random c,
 // 9.8 -> 6.7 ms on a random slice frame.  Two and three warps per quarter took 6.8
 // and 8.0 ms.  Claims of single pixels by idle lanes (no lockstep) executed 28 %
