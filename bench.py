@@ -339,7 +339,9 @@ def march_roofline(pass_ms, stats, peak, peak_basis, kernel, traffic, clocks=Non
     flops = sum(FLOPS_PER_ITER * stats[i % nf]["march_iters"] for i in range(len(march_ms)))
     achieved = flops / (sum(march_ms) * 1e-3) / 1e12
     roof = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3), "unit": "TFLOP/s",
-            "frac": round(achieved / peak, 4), "traffic": traffic, "kernel": kernel, "launches": len(march_ms),
+            "frac": round(achieved / peak, 4),
+            "traffic": None,  # recorded for the default form, below
+            "kernel": kernel, "launches": len(march_ms),
             "avg_launch_ms": round(sum(march_ms) / len(march_ms), 4), "flops_per_iter": FLOPS_PER_ITER,
             "peak_basis": peak_basis}
     if settles():  # most counts are proved, not iterated: no fraction of the FMA peak
