@@ -256,33 +256,43 @@ __device__ __forceinline__ void ray_w(const FrameT<T> &F, int x, int y, T (&w)[3
 }
 
 // FP64 entry and exit (tau) of a ray that crosses the box.  Only the faces that
-// can decide (within 1e-4 of the farthest entry or the nearest exit in FP32)
-// are intersected in FP64: one or two of three, and each needs one reciprocal,
-// formed by two Newton steps on an FP32 one (relative error 1e-7, 1e-14, then
-// rounding).  FP64 runs at 1/64 of the FP32 rate here: with the normalised
-// direction, three reciprocals and the whole clip a recheck took about 130 FP64
-// instructions, in this form about 85.
+// can decide are intersected in FP64, one or two of three as a rule, and each
+// needs one reciprocal, formed by two Newton steps on an FP32 one (relative error
+// 1e-7, 1e-14, then rounding).  A face can decide unless its FP32 parameter lies
+// behind another's by more than their rounding: 8 u of itself (the ray, its
+// reciprocal, the product), and |1/w| times 3 u of the face's and the eye's
+// coordinates, whose difference cancels where the eye is next to the face.  FP64
+// runs at 1/64 of the FP32 rate here: with the normalised direction, three
+// reciprocals and the whole clip a recheck took about 130 FP64 instructions, in
+// this form about 85.
 __device__ __forceinline__ void ray_clip64(const FrameDesc &fd, const double (&w)[3], double &t0, double &t1)
 {
     const FrameT<float> &f = fd.f;
     const FrameT<double> &F = fd.d;
-    float rw[3], in = 0.f, out = tinf<float>(), near[3], far[3];
+    constexpr float u = 5.9604645e-8f;
+    // per axis, the latest the entry and the earliest the exit can be
+    float rw[3], in_lo = 0.f, out_hi = tinf<float>(), entry[3], exit[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const float wf = (float)w[a];
         const bool flat = !(fabsf(wf) > 1e-30f);  // parallel to the slab, inside it
         rw[a] = 1.f / wf;
         const float p = (f.bmin[a] - f.eye[a]) * rw[a], q = (f.bmax[a] - f.eye[a]) * rw[a];
-        near[a] = flat ? -tinf<float>() : fminf(p, q);
-        far[a] = flat ? tinf<float>() : fmaxf(p, q);
-        in = fmaxf(in, near[a]);
-        out = fminf(out, far[a]);
+        const float near = fminf(p, q), far = fmaxf(p, q);
+        const float abs_r = 3.f * u * fabsf(rw[a]) * (fabsf(f.eye[a]) + fmaxf(fabsf(f.bmin[a]), fabsf(f.bmax[a])));
+        const float dn = fmaf(8.f * u, fabsf(near), abs_r), df = fmaf(8.f * u, fabsf(far), abs_r);
+        entry[a] = flat ? -tinf<float>() : near + dn;
+        exit[a] = flat ? tinf<float>() : far - df;
+        if (!flat) {
+            in_lo = fmaxf(in_lo, near - dn);
+            out_hi = fminf(out_hi, far + df);
+        }
     }
     t0 = 0.0;
     t1 = tinf<double>();
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const bool ci = near[a] >= in - 1e-4f * in, co = far[a] <= out + 1e-4f * fabsf(out);
+        const bool ci = !(entry[a] < in_lo), co = !(exit[a] > out_hi);  // an overflowed one is intersected
         if (ci || co) {
             double r = (double)rw[a];
             r = fma(r, fma(-w[a], r, 1.0), r);

@@ -1,0 +1,120 @@
+// bounds_probe.cu -- the render kernels' device functions behind the recheck, one
+// call per thread or warp, for tests/test_gpu_bounds.py: built beside libdqj
+// from the same headers, with the library's own per-frame constants.
+#include "../paper_2303_14827_gb300/csrc/render_common.cuh"
+#include "../paper_2303_14827_gb300/csrc/runtime.h"
+
+using namespace dqj;
+
+namespace {
+
+// t0, t1 (in units of the ray w) of ray_clip64 and the ray itself.
+__global__ void clip_kernel(const __grid_constant__ FrameDesc fd, const int *x, const int *y, int n, double *t0,
+                            double *t1, double *w)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double v[3];
+    ray_w<double>(fd.d, x[i], y[i], v);
+    ray_clip64(fd, v, t0[i], t1[i]);
+    for (int a = 0; a < 3; ++a) w[3 * i + a] = v[a];
+}
+
+// which: 0 count_bound64, 1 count_bound2, 2 FP64 evaluation, 3 count64.
+template <int SQ, int MOD>
+__global__ void count_kernel(const __grid_constant__ FrameDesc fd, int which, const double *zs, int n, int *count,
+                             int *certain)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double z[8];
+    for (int j = 0; j < 8; ++j) z[j] = zs[8 * i + j];
+    bool ok = true;
+    int c;
+    if (which == 0)
+        c = count_bound64<SQ, MOD>(fd, z, ok);
+    else if (which == 1)
+        c = count_bound2<SQ, MOD>(fd, z, ok);
+    else if (which == 2)
+        c = classify_scalar<double, SQ, MOD>(z, fd.d, fd.max_iter);
+    else
+        c = count64<SQ, MOD>(fd, z);
+    count[i] = c;
+    certain[i] = ok;
+}
+
+// March sample k of pixel (x, y): its FP64 count from its FP64 position, and
+// whether count_certain vouches for that count and for the next one.
+template <int SQ, int MOD, bool AXIS>
+__global__ void sample_kernel(const __grid_constant__ FrameDesc fd, const int *x, const int *y, const int *k, int n,
+                              int *count, int *right, int *wrong)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double z[8];
+    entry_point64(fd, make_int4(y[i] * fd.W + x[i], k[i] | (kMarchSample << 16), x[i] | (y[i] << 16), 0), z);
+    const int c = classify_scalar<double, SQ, MOD>(z, fd.d, fd.max_iter);
+    count[i] = c;
+    right[i] = count_certain<SQ, MOD, AXIS>(fd, x[i], y[i], k[i], c);
+    wrong[i] = count_certain<SQ, MOD, AXIS>(fd, x[i], y[i], k[i], c + 1);
+}
+
+FrameDesc frame_of(const dqj_params *p)
+{
+    FrameDesc fd;
+    derive_frame(*p, fd, 8, 8);
+    return fd;
+}
+
+int done()
+{
+    const cudaError_t e = cudaDeviceSynchronize();
+    return (int)(e != cudaSuccess ? e : cudaGetLastError());
+}
+
+}  // namespace
+
+extern "C" {
+
+int probe_clip(const dqj_params *p, const int *x, const int *y, int n, double *t0, double *t1, double *w)
+{
+    clip_kernel<<<(n + 127) / 128, 128>>>(frame_of(p), x, y, n, t0, t1, w);
+    return done();
+}
+
+int probe_count(const dqj_params *p, int which, const double *z, int n, int *count, int *certain)
+{
+    const FrameDesc fd = frame_of(p);
+    const int g = (n + 127) / 128;
+    switch (2 * p->square_mode + p->modulus_mode) {
+    case 0: count_kernel<0, 0><<<g, 128>>>(fd, which, z, n, count, certain); break;
+    case 1: count_kernel<0, 1><<<g, 128>>>(fd, which, z, n, count, certain); break;
+    case 2: count_kernel<1, 0><<<g, 128>>>(fd, which, z, n, count, certain); break;
+    default: count_kernel<1, 1><<<g, 128>>>(fd, which, z, n, count, certain); break;
+    }
+    return done();
+}
+
+int probe_samples(const dqj_params *p, const int *x, const int *y, const int *k, int n, int *count, int *right,
+                  int *wrong)
+{
+    const FrameDesc fd = frame_of(p);
+    const int g = (n + 127) / 128;
+    auto run = [&](auto sq, auto mod) {
+        if (fd.axis_slice)
+            sample_kernel<sq(), mod(), true><<<g, 128>>>(fd, x, y, k, n, count, right, wrong);
+        else
+            sample_kernel<sq(), mod(), false><<<g, 128>>>(fd, x, y, k, n, count, right, wrong);
+    };
+    using Z = std::integral_constant<int, 0>;
+    using O = std::integral_constant<int, 1>;
+    switch (2 * p->square_mode + p->modulus_mode) {
+    case 0: run(Z{}, Z{}); break;
+    case 1: run(Z{}, O{}); break;
+    case 2: run(O{}, Z{}); break;
+    default: run(O{}, O{}); break;
+    }
+    return done();
+}
+
+}  // extern "C"
