@@ -20,6 +20,17 @@ __global__ void clip_kernel(const __grid_constant__ FrameDesc fd, const int *x, 
     for (int a = 0; a < 3; ++a) w[3 * i + a] = v[a];
 }
 
+// FP64 slice points of march samples (entry_point64).
+__global__ void position_kernel(const __grid_constant__ FrameDesc fd, const int *x, const int *y, const int *k, int n,
+                                double *out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double z[8];
+    entry_point64(fd, make_int4(y[i] * fd.W + x[i], k[i] | (kMarchSample << 16), x[i] | (y[i] << 16), 0), z);
+    for (int j = 0; j < 8; ++j) out[8 * i + j] = z[j];
+}
+
 // which: 0 count_bound64, 1 count_bound2, 2 FP64 evaluation, 3 count64.
 template <int SQ, int MOD>
 __global__ void count_kernel(const __grid_constant__ FrameDesc fd, int which, const double *zs, int n, int *count,
@@ -79,6 +90,25 @@ extern "C" {
 int probe_clip(const dqj_params *p, const int *x, const int *y, int n, double *t0, double *t1, double *w)
 {
     clip_kernel<<<(n + 127) / 128, 128>>>(frame_of(p), x, y, n, t0, t1, w);
+    return done();
+}
+
+// The library's camera constants: forward, right and up, tan(fov_y / 2), aspect.
+void probe_camera(const dqj_params *p, double *out)
+{
+    const FrameDesc fd = frame_of(p);
+    for (int a = 0; a < 3; ++a) {
+        out[a] = fd.d.fwd[a];
+        out[3 + a] = fd.d.right[a];
+        out[6 + a] = fd.d.upv[a];
+    }
+    out[9] = fd.d.th;
+    out[10] = fd.d.aspect;
+}
+
+int probe_positions(const dqj_params *p, const int *x, const int *y, const int *k, int n, double *z)
+{
+    position_kernel<<<(n + 127) / 128, 128>>>(frame_of(p), x, y, k, n, z);
     return done();
 }
 

@@ -1,6 +1,7 @@
 """The recheck's device functions against plain FP64, called one by one through a
 probe library built from the same headers (bounds_probe.cu): the FP64 clip of a
-ray, the two orbit bounds, and the bound of a march sample's position."""
+ray, the positions of samples, the two orbit bounds, and the bound of a march
+sample's position."""
 import ctypes
 import os
 import subprocess
@@ -80,6 +81,53 @@ def test_ray_clip(probe, off, box):
                 bad = err > 8 * 2.0 ** -53 * np.abs(want[ok])
                 assert not bad.any(), (sides, int(bad.sum()), float(err.max()))
     assert tested > 20000
+
+
+def ray_points(s, cam, x, y, k, T):
+    """Slice points of march samples by the reference formula in type T, from the
+    library's own (FP64) camera constants, and which of the rays cross the box."""
+    t = {n: np.array(s[n], dtype=T) for n in ("eye", "box_min", "box_max", "slice_origin", "slice_basis")}
+    f, r, u = (cam[3 * a:3 * a + 3].astype(T) for a in range(3))
+    th, aspect = T(cam[9]), T(cam[10])
+    sx = (2 * (x.astype(T) + T(0.5)) / s["width"] - 1) * th * aspect
+    sy = (1 - 2 * (y.astype(T) + T(0.5)) / s["height"]) * th
+    d = f + sx[:, None] * r + sy[:, None] * u
+    d = d / np.sqrt((d * d).sum(1))[:, None]
+    with np.errstate(all="ignore"):
+        a, b = (t["box_min"] - t["eye"]) / d, (t["box_max"] - t["eye"]) / d
+    t0 = np.maximum(np.fmin(a, b).max(1), 0)
+    t1 = np.fmax(a, b).min(1)
+    tau = t0 + k.astype(T) * ((t1 - t0) / s["march_steps"])
+    return t["slice_origin"] + (t["eye"] + tau[:, None] * d) @ t["slice_basis"], t1 - t0 > 1e-3
+
+
+@pytest.mark.parametrize("eye", ([0.37, 0.23, 3.4], [2.3, 1.1, 2.6], [0.1, 0.2, 0.3]))
+@pytest.mark.parametrize("seed", (None, 1, 2))
+def test_sample_positions(probe, eye, seed):
+    # the recheck places its samples as closely as the reference formula in FP64
+    # does (rms over many samples; the two differ by sampling, a few per cent)
+    import torch
+    assert np.finfo(np.longdouble).nmant >= 63
+    rng = np.random.default_rng(23)
+    n = 60000
+    s = scenes.default_scene(width=1920, height=1080, march_steps=512, precision=1, eye=eye, target=[0.05, -0.11, 0.02])
+    if seed is not None:
+        s["slice_basis"] = scenes.random_slice_frame(np.random.default_rng(seed))
+    x, y, k = (rng.integers(0, m, n).astype(np.int32) for m in (1920, 1080, 513))
+    p = binding.make_params(s)
+    cam = np.empty(11)
+    probe.probe_camera(ctypes.byref(p), ctypes.c_void_p(cam.ctypes.data))
+    exact, ok = ray_points(s, cam, x, y, k, np.longdouble)
+    plain, _ = ray_points(s, cam, x, y, k, np.float64)
+    z = torch.empty(n, 8, dtype=torch.float64, device="cuda")
+    dx, dy, dk = dev(x), dev(y), dev(k)
+    assert probe.probe_positions(ctypes.byref(p), ptr(dx), ptr(dy), ptr(dk), n, ptr(z)) == 0
+
+    def rms(v):
+        return float(np.sqrt((((v - exact)[ok]) ** 2).sum(1).mean()))
+
+    assert ok.sum() > n // 8
+    assert rms(z.cpu().numpy()) <= 1.05 * rms(plain)
 
 
 def classify(probe, p, which, z):
