@@ -911,9 +911,20 @@ constexpr int kQStage = 320;
 // its distance from R^2 never falls within a recheck band.
 constexpr float kFarT = 1e18f;
 
+// Entry `at` of the recheck queue.  One beyond the queue's capacity is counted as
+// an overflow, and its pixel is re-rendered in FP64 instead.
+__device__ __forceinline__ void queue_entry(const FrameDesc &fd, const Scratch &sc, unsigned at, int4 e)
+{
+    if (at < sc.queue_cap) {
+        sc.queue[at] = e;
+    } else {
+        atomicAdd(&sc.ctr->stats[7], 1ull);
+        mark_dirty(fd, sc, e.x);
+    }
+}
+
 // Append a warp's staged entries qs[0, qn) to the recheck queue (qn warp-uniform)
-// and count those from `counted` on as rechecks; entries beyond the queue's capacity re-render
-// their pixel in FP64.
+// and count those from `counted` on as rechecks.
 __device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch &sc, const int4 *qs, int qn,
                                              int counted)
 {
@@ -926,22 +937,9 @@ __device__ __forceinline__ void flush_staged(const FrameDesc &fd, const Scratch 
     }
     base = __shfl_sync(kFull, base, 0);
     for (int i = lane; i < qn; i += 32) {
-        const int4 e = qs[i];
-        if (base + (unsigned)i < sc.queue_cap) {
-            sc.queue[base + i] = e;
-        } else {
-            atomicAdd(&sc.ctr->stats[7], 1ull);
-            mark_dirty(fd, sc, e.x);
-        }
+        queue_entry(fd, sc, base + (unsigned)i, qs[i]);
     }
     __syncwarp();
-}
-
-// recheck_entry out of line, for entries that find the queue full.
-template <int SQ, int MOD>
-__device__ __noinline__ void recheck_entry_call(const FrameDesc &fd, const Scratch &sc, int4 e)
-{
-    recheck_entry<SQ, MOD>(fd, sc, e);
 }
 
 // Recheck of a warp's staged entries qs[0, qn) (qn warp-uniform), counted as
@@ -975,11 +973,7 @@ __device__ __forceinline__ int recheck_staged(const FrameDesc &fd, const Scratch
             const int4 v = qs[out + lane];
             unsigned at = 0;
             if (lane == 0) at = atomicAdd(&sc.ctr->queue_count, 32u);
-            at = __shfl_sync(kFull, at, 0) + lane;
-            if (at < sc.queue_cap)
-                sc.queue[at] = v;
-            else
-                recheck_entry_call<SQ, MOD>(fd, sc, v);
+            queue_entry(fd, sc, __shfl_sync(kFull, at, 0) + lane, v);
             __syncwarp();
         }
     }
@@ -1025,15 +1019,7 @@ __device__ __forceinline__ void flush_rest(const FrameDesc &fd, const Scratch &s
     unsigned base = 0;
     if (lane == 0 && qn > 0) base = atomicAdd(&sc.ctr->queue_count, (unsigned)qn);
     base = __shfl_sync(kFull, base, 0);
-    if (lane < qn) {
-        const int4 e = qs[lane];
-        if (base + (unsigned)lane < sc.queue_cap) {
-            sc.queue[base + lane] = e;
-        } else {
-            atomicAdd(&sc.ctr->stats[7], 1ull);
-            mark_dirty(fd, sc, e.x);
-        }
-    }
+    if (lane < qn) queue_entry(fd, sc, base + (unsigned)lane, qs[lane]);
     __syncwarp();
 }
 

@@ -70,6 +70,17 @@ __global__ void sample_kernel(const __grid_constant__ FrameDesc fd, const int *x
     wrong[i] = count_certain<SQ, MOD, AXIS>(fd, x[i], y[i], k[i], c + 1);
 }
 
+// One warp: n staged entries of march samples whose FP32 count is wrong by one,
+// against a queue of `cap` entries; ctr, flags and list as in a frame's scratch.
+__global__ void staged_kernel(const __grid_constant__ FrameDesc fd, Scratch sc, const int4 *entries, int n)
+{
+    __shared__ int4 qs[kQStage];
+    for (int i = threadIdx.x; i < n; i += 32) qs[i] = entries[i];
+    __syncwarp();
+    const int left = recheck_staged<0, 0, true>(fd, sc, qs, n, 0);
+    flush_rest(fd, sc, qs, left);
+}
+
 FrameDesc frame_of(const dqj_params *p)
 {
     FrameDesc fd;
@@ -145,6 +156,31 @@ int probe_samples(const dqj_params *p, const int *x, const int *y, const int *k,
     default: run(O{}, O{}); break;
     }
     return done();
+}
+
+// stats (DQJ_NSTATS), queue_count and dirty_count of the scratch after n <= 320
+// staged entries; queue: room for `cap` entries, flags and list: one per pixel.
+int probe_staged(const dqj_params *p, const int *entries, int n, int *queue, int cap, unsigned *flags, int *list,
+                 unsigned long long *counters)
+{
+    FrameDesc fd = frame_of(p);
+    fd.epoch = 1;
+    Scratch sc{};
+    sc.ctr = reinterpret_cast<Counters *>(counters);
+    sc.queue = reinterpret_cast<int4 *>(queue);
+    sc.queue_cap = (uint32_t)cap;
+    sc.dirty_flag = flags;
+    sc.dirty_list = list;
+    sc.dirty_cap = (uint32_t)(fd.W * fd.H);
+    staged_kernel<<<1, 32>>>(fd, sc, reinterpret_cast<const int4 *>(entries), n);
+    return done();
+}
+
+int probe_counter_offsets(int *queue_count, int *dirty_count)
+{
+    *queue_count = (int)offsetof(Counters, queue_count);
+    *dirty_count = (int)offsetof(Counters, dirty_count);
+    return (int)sizeof(Counters);
 }
 
 }  // extern "C"

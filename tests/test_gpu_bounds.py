@@ -1,7 +1,8 @@
 """The recheck's device functions against plain FP64, called one by one through a
 probe library built from the same headers (bounds_probe.cu): the FP64 clip of a
-ray, the positions of samples, the two orbit bounds, and the bound of a march
-sample's position."""
+ray, the positions of samples, the two orbit bounds, the bound of a march
+sample's position, and what becomes of staged samples that find the recheck queue
+full."""
 import ctypes
 import os
 import subprocess
@@ -211,3 +212,33 @@ def test_sample_certain(probe, square, modulus):
             assert not o[2].any(), (axis, view, int(o[2].sum()))
             right += int(o[1].sum())
     assert right > n  # and it vouches for many of the right ones
+
+
+@pytest.mark.parametrize("n", (1, 31, 32, 33, 64, 320))
+@pytest.mark.parametrize("cap", (0, 1, 40, 1000))
+def test_full_queue(probe, n, cap):
+    # every staged sample left over is in the queue, or counted as an overflow
+    # and its pixel listed for the FP64 re-render
+    import torch
+    w, h = 64, 45
+    p = scene_params(width=w, height=h, precision=1, march_steps=512)
+    px = np.arange(n, dtype=np.int32) * 7
+    e = np.stack([px, (100 + 0 * px) | (31 << 16), px % w | (px // w << 16), 0 * px + 99], 1).astype(np.int32)
+    entries = dev(e)
+    queue = torch.zeros(max(cap, 1), 4, dtype=torch.int32, device="cuda")
+    flags = torch.zeros(w * h, dtype=torch.int32, device="cuda")
+    listed = torch.full((w * h,), -1, dtype=torch.int32, device="cuda")
+    oq, od = ctypes.c_int32(), ctypes.c_int32()
+    size = probe.probe_counter_offsets(ctypes.byref(oq), ctypes.byref(od))
+    ctr = torch.zeros(size, dtype=torch.uint8, device="cuda")
+    assert probe.probe_staged(ctypes.byref(p), ptr(entries), n, ptr(queue), cap, ptr(flags), ptr(listed), ptr(ctr)) == 0
+    raw = ctr.cpu().numpy()
+    stats = raw[:80].view(np.int64)
+    queued = min(cap, n)
+    assert stats[4] == n
+    assert raw[oq.value:oq.value + 4].view(np.uint32)[0] == n
+    assert stats[7] == n - queued
+    dirty = int(raw[od.value:od.value + 4].view(np.uint32)[0])
+    q = queue.cpu().numpy()[:queued, 0]
+    d = listed.cpu().numpy()[:dirty]
+    assert dirty == n - queued and sorted(np.concatenate([q, d]).tolist()) == px.tolist()
