@@ -267,20 +267,22 @@ __device__ __forceinline__ int classify_scalar_axis(T (&z)[8], const FrameT<T> &
 {
     T sp = dfma(z[2], z[2], z[1] * z[1]);
     if (max_iter < 1) return 0;
-    if (dq_iter_axis_first<T, MOD>(z, z, sp, F.c) > F.R2) return 1;
+    if (!bounded(dq_iter_axis_first<T, MOD>(z, z, sp, F.c), F.R2)) return 1;
 #pragma unroll 1
     for (int n = 2; n <= max_iter; ++n)
-        if (dq_iter<T, SQ, MOD>(z, z, sp, F.c) > F.R2) return n;
+        if (!bounded(dq_iter<T, SQ, MOD>(z, z, sp, F.c), F.R2)) return n;
     return 0;
 }
 
+// Escape count of one sample (0: bounded for max_iter steps).  As in the lockstep
+// forms, a modulus that is not a number has escaped.
 template <typename T, int SQ, int MOD>
 __device__ __forceinline__ int classify_scalar(T (&z)[8], const FrameT<T> &F, int max_iter)
 {
     T sp = dq_sp<T>(z);
 #pragma unroll 1
     for (int n = 1; n <= max_iter; ++n)
-        if (dq_iter<T, SQ, MOD>(z, z, sp, F.c) > F.R2) return n;
+        if (!bounded(dq_iter<T, SQ, MOD>(z, z, sp, F.c), F.R2)) return n;
     return 0;
 }
 
