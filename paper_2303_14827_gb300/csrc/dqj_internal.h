@@ -82,9 +82,10 @@ struct alignas(16) FrameDesc {
     int32_t march_samples;  // paired FP32 march: samples of each ray per round (1, 2)
     // settled blocks (settle.cuh): thresholds of a proved escape and of a proved
     // bounded step (R^2 and the recheck margin, with room for rounding), |c|,
-    // |slice origin| + |eye|, and whether blocks are settled (march_settles)
+    // |slice origin| + |eye|, and whether the march settles blocks (settle_pays)
     float settle_hi, settle_lo, settle_cn, settle_an;
     int32_t settle;
+    int32_t bounds;   // orbit bounds may decide a sample (bounds_hold)
     double inv_n;     // 1 / N
 };
 

@@ -385,6 +385,8 @@ __device__ __forceinline__ int count_bound(const FrameDesc &fd, float (&z)[8], f
 {
     const FrameT<float> &F = fd.f;
     constexpr float u = 5.9604645e-8f;
+    certain = false;
+    if (!fd.bounds) return 0;
     const float hi = F.R2 * (1.f + 2.f * u), lo = F.R2 * (1.f - 2.f * u);
     float sp = dq_sp<float>(z);
     float r2 = fmaf(z[0], z[0], sp), d2 = fmaf(z[7], z[7], fmaf(z[6], z[6], fmaf(z[5], z[5], z[4] * z[4])));
@@ -470,6 +472,8 @@ __device__ __forceinline__ int count_bound2(const FrameDesc &fd, const double (&
 {
     constexpr float u = 5.9604645e-8f;
     constexpr int nc = MOD == 0 ? 8 : 4;  // components that a test can see
+    certain = false;
+    if (!fd.bounds) return 0;
     const float R2 = fd.f.R2, hi = R2 * (1.f + 2.f * u), lo = R2 * (1.f - 2.f * u);
     float zh[8], zl[8];
 #pragma unroll
@@ -812,7 +816,7 @@ __device__ __forceinline__ void fixup_pixels(const FrameDesc &fd, const Scratch 
             const bool part = k <= fd.N;
             // the ray's settled samples (blocks of 16, chunks of 512: see
             // settle.cuh) have their counts; the others are classified
-            if (k0 % kSettleChunk == 0) {
+            if (fd.bounds && k0 % kSettleChunk == 0) {
                 const int ke = min(k0 + kSettleChunk, fd.N + 1);
                 w = fd.axis_slice ? settle_chunk<SQ, MOD, true>(fd, box, k0, ke, kSettlePairs)
                                   : settle_chunk<SQ, MOD, false>(fd, box, k0, ke, kSettlePairs);

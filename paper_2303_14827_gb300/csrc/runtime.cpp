@@ -235,6 +235,12 @@ static bool settle_pays(const dqj_params &p, int tile_w, int tile_h)
     return width <= (p.precision == DQJ_FP64 ? 0.25 : 0.022);
 }
 
+// Whether the FP32 bounds of an orbit (settle.cuh, count_bound) hold at this
+// escape radius.  Their rounding terms are relative to the iterates: far below R^2
+// = 1e-24 squares underflow instead (R = 1e-22: R^2 has three bits left in FP32),
+// far above 1e30 they overflow.
+static bool bounds_hold(double R2) { return R2 >= 1e-24 && R2 <= 1e30; }
+
 void derive_frame(const dqj_params &p, FrameDesc &fd, int tile_w, int tile_h)
 {
     std::memset(&fd, 0, sizeof fd);
@@ -332,7 +338,8 @@ void derive_frame(const dqj_params &p, FrameDesc &fd, int tile_w, int tile_h)
         fd.settle_lo = (float)(F.R2 * (1.0 - 2e-5) - m);
         fd.settle_cn = (float)norm(p.c, 8);
         fd.settle_an = (float)(norm(p.slice_origin, 8) + norm(p.eye, 3));
-        fd.settle = march_settles() && settle_pays(p, tile_w, tile_h);
+        fd.bounds = bounds_hold(F.R2);
+        fd.settle = fd.bounds && march_settles() && settle_pays(p, tile_w, tile_h);
     }
 }
 

@@ -1,7 +1,9 @@
-"""Calls at the ends of what the parameters allow: boxes whose samples overflow."""
+"""Calls at the ends of what the parameters allow: boxes whose samples overflow, and
+escape radii below what FP32 squares resolve."""
 import numpy as np
 import pytest
 
+import oracle
 from paper_2303_14827_gb300 import binding, scenes
 from parity import to_numpy
 
@@ -29,3 +31,21 @@ def test_overflowing_samples_escape(square, modulus, precision, half, general):
         binding.dqj_voxelize(r.ctx, s, n, occ, cnt, None, torch.cuda.current_stream().cuda_stream)
         torch.cuda.synchronize()
         assert not occ.any() and bool((cnt == 1).all())
+
+
+@pytest.mark.parametrize("radius", (1e-22, 1e-19, 1e-16, 1e-11))
+def test_fp64_tiny_radius(radius):
+    # |zeta_1|^2 against R^2 = 1e-44 .. 1e-22: subnormal or nearly so in FP32
+    u = radius ** 0.5
+    c = [0.3 * radius, -0.2 * radius, 0.1 * radius, 0.0, 0.1 * radius, 0.0, 0.0, 0.05 * radius]
+    s = scenes.default_scene(width=72, height=40, precision=2, escape_radius=radius, c=c, normal_h=1e-4 * u,
+                             box_min=[-2 * u] * 3, box_max=[2 * u] * 3, eye=[0.4 * u, 0.3 * u, 3.5 * u],
+                             target=[0.0, 0.1 * u, 0.0])
+    with binding.Renderer(0) as r:
+        g = to_numpy(r.render(s), 72, 40)
+    o = oracle.render(s)
+    hg, ho = np.isfinite(g["depth"]), np.isfinite(o["depth"])
+    assert 100 < ho.sum() < 2800
+    assert np.array_equal(hg, ho) and np.array_equal(g["iter"], o["iter"])
+    # a bracket is 3 u / 256 / 2^8 long; a decision within FP64 rounding moves it by one last place
+    assert np.abs(g["depth"][ho].astype(np.float64) - o["depth"][ho]).max() <= 1e-6 * 4 * u
