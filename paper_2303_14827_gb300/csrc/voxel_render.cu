@@ -98,7 +98,7 @@ __device__ __forceinline__ bool walk_setup(const FrameDesc &fd, const GridGeom &
     const double il = rsqrt(W.d[0] * W.d[0] + W.d[1] * W.d[1] + W.d[2] * W.d[2]);
     double tb[3];
     float df[3], te[3], in = -tinf<float>(), mid = -tinf<float>(), out = tinf<float>();
-    bool in_box = true;
+    bool in_box = true, finite = true;
     W.tol = 0.f;
     W.axis = -1;
 #pragma unroll
@@ -135,17 +135,21 @@ __device__ __forceinline__ bool walk_setup(const FrameDesc &fd, const GridGeom &
         // spare), so when the two nearest planes differ by more than the sum of the
         // bounds the FP32 order is the FP64 order; otherwise the choice is FP64's.
         // An axis whose FP32 plane distances overflow (|d| below ~1e-38) crosses no
-        // cell plane inside the box, like an axis the ray runs parallel to.
+        // cell plane inside the box, like an axis the ray runs parallel to; whether
+        // the ray meets the box at all is then left to the FP64 distances.
         const bool cross = isfinite(W.d32[a]) && isfinite(W.b32[a]);
         W.E[a] = cross ? 4.76837158203125e-7f * ((float)g * fabsf(W.d32[a]) + fabsf(W.b32[a])) : 0.f;
         W.tol += W.E[a];
-        if (!cross) W.s[a] = 0;
+        if (!cross) {
+            W.s[a] = 0;
+            finite = false;
+        }
     }
     W.t_in = in > 0.f ? (W.axis == 0 ? (W.s[0] > 0 ? W.b64[0] : tb[0])
                                      : (W.axis == 1 ? (W.s[1] > 0 ? W.b64[1] : tb[1]) : (W.s[2] > 0 ? W.b64[2] : tb[2])))
                       : 0.0;
     bool crosses = in_box;
-    if (!(in - mid > W.tol && fabsf(in) > W.tol && out - fmaxf(in, 0.f) > W.tol)) {
+    if (!(finite && in - mid > W.tol && fabsf(in) > W.tol && out - fmaxf(in, 0.f) > W.tol)) {
         // too close for FP32: entry and exit by the FP64 distances
         double t0 = -tinf<double>(), t1 = tinf<double>();
         W.axis = -1;

@@ -1,5 +1,6 @@
-"""Calls at the ends of what the parameters allow: boxes whose samples overflow, and
-escape radii below what FP32 squares resolve."""
+"""Calls at the ends of what the parameters allow: boxes whose samples overflow,
+escape radii below what FP32 squares resolve, and rays that run almost parallel
+to a slab they lie outside of."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,22 @@ def test_fp64_tiny_radius(radius):
     assert np.array_equal(hg, ho) and np.array_equal(g["iter"], o["iter"])
     # a bracket is 3 u / 256 / 2^8 long; a decision within FP64 rounding moves it by one last place
     assert np.abs(g["depth"][ho].astype(np.float64) - o["depth"][ho]).max() <= 1e-6 * 4 * u
+
+
+@pytest.mark.parametrize("g", (8, 24, 100))
+@pytest.mark.parametrize("side", (1.0, -1.0))
+def test_voxel_ray_beside_the_grid(g, side):
+    # direction 2e-41 along y, the eye outside the box on y: no ray meets the grid
+    import torch
+    s = scenes.default_scene(width=64, height=1, eye=[5.0, 1e-40, 0.0], target=[0.0, 0.0, 0.0],
+                             box_min=[-2.0, -2.0 if side > 0 else 1.0, -2.0],
+                             box_max=[2.0, -1.0 if side > 0 else 2.0, 2.0])
+    occ = np.ones((g, g, g), dtype=np.uint8)
+    assert not np.isfinite(oracle.voxel_render(s, occ)["depth"]).any()
+    with binding.Renderer(0) as r:
+        t = binding.alloc_outputs(64, 1, stats=False)
+        d_occ = torch.from_numpy(occ.reshape(-1)).cuda()
+        binding.dqj_render_voxels(r.ctx, s, g, d_occ, binding.outputs_of(t), torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        out = to_numpy(t, 64, 1)
+    assert np.all(np.isinf(out["depth"])) and np.all(out["iter"] == 0)
