@@ -496,6 +496,16 @@ __global__ void __launch_bounds__(kBlock) voxel_mip_kernel(const uint8_t *__rest
 // the search of its first cell.
 int mip_shift(int g) { return g >= 96 ? 3 : (g >= 24 ? 2 : 0); }
 
+// Allocates from the stream's pool without disturbing a capture under way on
+// another stream or thread: in the default mode the pool's calls are not allowed
+// beside one (they fail and invalidate it), although nothing here is captured.
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { swap(); }
+    ~BesideCaptures() { swap(); }
+    void swap() { (void)cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 // The context's pool for block occupancies: it keeps its memory between calls (at
 // most 2 MiB for each call in flight), until dqj_destroy.
 bool ensure_mip_pool(dqj_ctx *ctx)
@@ -569,6 +579,7 @@ extern "C" dqj_status dqj_render_voxels(dqj_ctx *ctx, const dqj_params *p, int32
         uint8_t *mip = nullptr;
         const int gb = shift ? (grid_n + (1 << shift) - 1) >> shift : 0;
         const uint32_t blocks = (uint32_t)gb * (uint32_t)gb * (uint32_t)gb;
+        const BesideCaptures relaxed;
         if (shift) {
             (void)cudaGetLastError();
             cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
