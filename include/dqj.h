@@ -54,7 +54,12 @@ enum {
     DQJ_FP32_RECHECK = 1, /* FP32, samples within recheck_margin of R^2 decided at
                              FP64 accuracy on the GPU (a rounding bound, or FP64);
                              a pixel whose decision differs is re-rendered so        */
-    DQJ_FP64 = 2          /* FP64 throughout                                         */
+    DQJ_FP64 = 2          /* FP64 throughout: positions, depths, normals and shading in
+                             FP64, every sample's escape count the one FP64 evaluation
+                             gives.  A count that a rounding bound of an FP32 or
+                             two-float orbit proves is not evaluated again; with the
+                             environment variable DQJ_BOUNDS=0 every count is, here and
+                             in DQJ_FP32_RECHECK's rechecks and re-renders            */
 };
 
 /* dqj_params.square_mode (Method, "Dual-Quaternion Julia Sets") */

@@ -85,7 +85,8 @@ struct alignas(16) FrameDesc {
     // |slice origin| + |eye|, and whether the march settles blocks (settle_pays)
     float settle_hi, settle_lo, settle_cn, settle_an;
     int32_t settle;
-    int32_t bounds;   // orbit bounds may decide a sample (bounds_hold)
+    int32_t bounds;   // orbit bounds may decide a sample (bounds_hold, bounds_decide)
+    int32_t blocks;   // and settled blocks stand for their samples outside the march too
     double inv_n;     // 1 / N
 };
 
@@ -142,5 +143,9 @@ int march_split(const FrameDesc &fd, int num_sms);
 // or 1.  All forms give the same results.
 int march_samples_per_round();
 bool march_settles();
+// Whether rounding bounds decide samples at all: yes unless DQJ_BOUNDS = 0 (read
+// once per process), when every sample is iterated in its own precision and every
+// recheck in FP64.  Both give the same results.
+bool bounds_decide();
 
 }  // namespace dqj

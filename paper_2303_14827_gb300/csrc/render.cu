@@ -18,7 +18,16 @@ int march_samples_env()  // DQJ_MARCH_SAMPLES, or -1
 
 int march_samples_per_round() { return march_samples_env() == 1 ? 1 : 2; }
 
-bool march_settles() { return march_samples_env() != 0 && march_samples_env() != 1; }
+bool bounds_decide()
+{
+    static const bool on = [] {
+        const char *e = std::getenv("DQJ_BOUNDS");
+        return !(e && e[0] == '0');
+    }();
+    return on;
+}
+
+bool march_settles() { return bounds_decide() && march_samples_env() != 0 && march_samples_env() != 1; }
 
 int march_split(const FrameDesc &fd, int num_sms)
 {

@@ -816,7 +816,7 @@ __device__ __forceinline__ void fixup_pixels(const FrameDesc &fd, const Scratch 
             const bool part = k <= fd.N;
             // the ray's settled samples (blocks of 16, chunks of 512: see
             // settle.cuh) have their counts; the others are classified
-            if (fd.bounds && k0 % kSettleChunk == 0) {
+            if (fd.blocks && k0 % kSettleChunk == 0) {
                 const int ke = min(k0 + kSettleChunk, fd.N + 1);
                 w = fd.axis_slice ? settle_chunk<SQ, MOD, true>(fd, box, k0, ke, kSettlePairs)
                                   : settle_chunk<SQ, MOD, false>(fd, box, k0, ke, kSettlePairs);

@@ -338,8 +338,9 @@ void derive_frame(const dqj_params &p, FrameDesc &fd, int tile_w, int tile_h)
         fd.settle_lo = (float)(F.R2 * (1.0 - 2e-5) - m);
         fd.settle_cn = (float)norm(p.c, 8);
         fd.settle_an = (float)(norm(p.slice_origin, 8) + norm(p.eye, 3));
-        fd.bounds = bounds_hold(F.R2);
-        fd.settle = fd.bounds && march_settles() && settle_pays(p, tile_w, tile_h);
+        fd.bounds = bounds_decide() && bounds_hold(F.R2);
+        fd.blocks = fd.bounds && march_settles();
+        fd.settle = fd.blocks && settle_pays(p, tile_w, tile_h);
     }
 }
 

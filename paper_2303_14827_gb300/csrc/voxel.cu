@@ -495,7 +495,7 @@ cudaError_t launch_voxels_t(const FrameDesc &fd, const VoxelArgs &args, cudaStre
     }
     const bool re = fd.precision == DQJ_FP32_RECHECK;
     const int axis = fd.axis_slice ? 1 : 0;
-    if (args.g >= kBrickGrid && fd.bounds && march_settles()) {
+    if (args.g >= kBrickGrid && fd.blocks) {
         // bricks per claim: 32 or 16 (one settle pass of a warp) where every resident
         // warp gets several claims of that, else four (one pass over their sub-bricks)
         VoxelArgs va = args;

@@ -81,6 +81,31 @@ __global__ void staged_kernel(const __grid_constant__ FrameDesc fd, Scratch sc, 
     flush_rest(fd, sc, qs, left);
 }
 
+// Samples of the frame's 8 x 8 tiles [0, tiles) that the settled blocks cover.
+template <int SQ, int MOD, bool AXIS>
+__global__ void settled_kernel(const __grid_constant__ FrameDesc fd, int tiles, unsigned long long *out)
+{
+    __shared__ TileBox box;
+    const int lane = threadIdx.x, tile = blockIdx.x;
+    const int x0 = tile % fd.tiles_x * fd.tile_w, y0 = tile / fd.tiles_x * fd.tile_h;
+    float d[2][3], ti[2] = {0.f, 0.f}, to[2] = {0.f, 0.f};
+    bool act[2];
+    for (int s = 0; s < 2; ++s) {
+        const int slot = lane + 32 * s, x = x0 + slot % fd.tile_w, y = y0 + slot / fd.tile_w;
+        act[s] = x < fd.W && y < fd.H && camera_clip<float>(fd.f, fd.W, fd.H, x, y, d[s], ti[s], to[s]);
+    }
+    tile_box(fd, act[0], d[0], ti[0], to[0], act[1], d[1], ti[1], to[1], box);
+    unsigned samples = 0;
+    for (int kc = 0; kc <= fd.N; kc += kSettleChunk) {
+        const int ke = min(kc + kSettleChunk, fd.N + 1), pairs = settle_pairs(ke - kc);
+        const unsigned w = ke - kc > kSettleMin ? settle_chunk<SQ, MOD, AXIS>(fd, box, kc, ke, pairs) : 0u;
+        for (int p = 0; p < pairs; ++p)
+            if ((w >> (4 * p)) & 15u) samples += (unsigned)max(0, min(2, ke - (kc + 2 * (pairs * lane + p))));
+    }
+    samples = __reduce_add_sync(kFull, samples);
+    if (lane == 0) atomicAdd(out, (unsigned long long)samples);
+}
+
 FrameDesc frame_of(const dqj_params *p)
 {
     FrameDesc fd;
@@ -181,6 +206,29 @@ int probe_counter_offsets(int *queue_count, int *dirty_count)
     *queue_count = (int)offsetof(Counters, queue_count);
     *dirty_count = (int)offsetof(Counters, dirty_count);
     return (int)sizeof(Counters);
+}
+
+// Whether the frame settles blocks, and the samples they cover (all tiles).
+int probe_settled(const dqj_params *p, int *settles, unsigned long long *samples)
+{
+    const FrameDesc fd = frame_of(p);
+    *settles = fd.settle;
+    const int tiles = fd.tiles_x * fd.tiles_y;
+    auto run = [&](auto sq, auto mod) {
+        if (fd.axis_slice)
+            settled_kernel<sq(), mod(), true><<<tiles, 32>>>(fd, tiles, samples);
+        else
+            settled_kernel<sq(), mod(), false><<<tiles, 32>>>(fd, tiles, samples);
+    };
+    using Z = std::integral_constant<int, 0>;
+    using O = std::integral_constant<int, 1>;
+    switch (2 * p->square_mode + p->modulus_mode) {
+    case 0: run(Z{}, Z{}); break;
+    case 1: run(Z{}, O{}); break;
+    case 2: run(O{}, Z{}); break;
+    default: run(O{}, O{}); break;
+    }
+    return done();
 }
 
 }  // extern "C"
