@@ -28,7 +28,6 @@ struct VoxelArgs {
     uint32_t segs_per_row;                 // FP32, row segments
     uint64_t nsegs;
     uint32_t bricks_x, bricks_y, nbricks;  // FP32, bricks along x, along y, in all
-    uint32_t per_claim;                    // bricks claimed at a time, 1..32
     float radius;                          // |slice origin| + largest |corner| of the box
     int32_t wide;                          // rows of 16 cells are 16-byte aligned in occ and counts
     uint8_t *occ;       // g^3 or NULL
@@ -190,18 +189,20 @@ __global__ void __launch_bounds__(kBlock, 5) voxel2_kernel(const __grid_constant
 
 // Bricks against 32 x 2 row segments, FP32, axis / random slice (ms): 256^3 0.105 /
 // 0.143 against 0.092 / 0.135, 300^3 0.141 / 0.192 against 0.130 / 0.199, 333^3 0.166 /
-// 0.225 against 0.166 / 0.253, 400^3 0.19 / 0.29 against 0.25 / 0.40, 1024^3 1.97 /
-// 2.95 against 3.42 / 5.73: coarse bricks settle too seldom to pay for the bound.
+// 0.225 against 0.166 / 0.253, 400^3 0.16 / 0.27 against 0.25 / 0.40, 1024^3 1.67 /
+// 2.83 against 3.42 / 5.73: coarse bricks settle too seldom to pay for the bound.
 constexpr int kBrickGrid = 336;
 constexpr int kBrickX = 16, kBrickY = 8, kBrickZ = 4;  // a brick; its eight sub-bricks are half as long each way
+constexpr uint32_t kBrickClaim = 4;                     // bricks a warp claims: a sub-brick per lane
 
-// The count (15: inside) shared by the cells [x, x + nx) x [y, y + ny) x [z, z + nz) (clipped to
-// the grid), or 0 when the bound does not prove one.
+// The count (15: inside) shared by the cells of the sub-brick at (x, y, z) (clipped
+// to the grid), or 0 when the bound does not prove one.
 template <int SQ, int MOD, bool AXIS>
 __device__ __forceinline__ int settle_cells(const FrameDesc &fd, const VoxelArgs &va, const float (&step)[3], int x,
-                                            int y, int z, int nx, int ny, int nz)
+                                            int y, int z)
 {
-    const int lo[3] = {x, y, z}, n[3] = {min(nx, va.g - x), min(ny, va.g - y), min(nz, va.g - z)};
+    const int lo[3] = {x, y, z};
+    const int n[3] = {min(kBrickX / 2, va.g - x), min(kBrickY / 2, va.g - y), min(kBrickZ / 2, va.g - z)};
     const float rho = 4e-6f * va.radius, e1 = 8e-6f * va.radius * va.radius;
     float p[3], h[3];
 #pragma unroll
@@ -225,13 +226,15 @@ __device__ __forceinline__ void fill_row16(const VoxelArgs &va, uint32_t lin, in
     }
 }
 
-// Grids of kBrickGrid cells a side or more (see the head of this file).  A claim's bricks are
-// settled one per lane, then the sub-bricks of the bricks left over, four bricks
-// at a time; lane b's word holds the counts of brick b's sub-bricks, four bits
-// each.  1024^3 (default constant): nine in ten sub-bricks settle
-// (inside ones too), 3.42 -> 1.97 ms; the 3.2 GB written take 0.47 ms at the
-// measured copy rate.  What is left is the classification of the others, whose
-// cells run 8 to max_iter steps.
+// Grids of kBrickGrid cells a side or more (see the head of this file).  A claim is
+// four bricks, whose 32 sub-bricks are settled one per lane.  Larger claims, whole
+// bricks tried first, bounded fewer boxes but left the warps unequal shares; they
+// were slower at every size (default c / random slice / random c, ms): 512^3 0.275 /
+// 0.473 / 0.189 with four bricks, 0.334 / 0.585 / 0.262 with 16, 0.404 / 0.714 / 0.280
+// with 32; 1024^3 1.68 / 2.80 / 1.33, 1.89 / 2.94 / 1.75, 1.95 / 2.93 / 1.87.
+// 1024^3 (default constant): nine in ten sub-bricks settle (inside ones too), 3.42 ->
+// 1.67 ms; the 3.2 GB written take 0.47 ms at the measured copy rate.  What is left
+// is the classification of the others, whose cells run 8 to max_iter steps.
 template <int SQ, int MOD, bool RECHECK, bool AXIS>
 __global__ void __launch_bounds__(kBlock, 5) voxel_brick_kernel(const __grid_constant__ FrameDesc fd, const VoxelArgs va)
 {
@@ -246,56 +249,36 @@ __global__ void __launch_bounds__(kBlock, 5) voxel_brick_kernel(const __grid_con
     unsigned long long iters = 0, inside_n = 0, rechecks = 0, cells = 0;
     for (;;) {
         uint32_t first = 0;
-        if (lane == 0) first = atomicAdd(&va.ctr->tile_next, va.per_claim);
+        if (lane == 0) first = atomicAdd(&va.ctr->tile_next, kBrickClaim);
         first = __shfl_sync(kFull, first, 0);
         if (first >= va.nbricks) break;
-        const int nb = (int)min(va.per_claim, va.nbricks - first);
-        // lane b: brick first + b
+        const int nb = (int)min(kBrickClaim, va.nbricks - first);
+        // lane 8 b + s: sub-brick s of brick first + b; w: the counts of the lane's
+        // brick, four bits a sub-brick
         int bx, by, bz;
+        unsigned w;
         {
-            const uint32_t id = first + (uint32_t)min(lane, nb - 1), row = id / va.bricks_x;
+            const uint32_t id = first + (uint32_t)min(lane >> 3, nb - 1), row = id / va.bricks_x;
             bx = (int)(id - row * va.bricks_x) * kBrickX;
             bz = (int)(row / va.bricks_y);
             by = (int)(row - (uint32_t)bz * va.bricks_y) * kBrickY;
             bz *= kBrickZ;
-        }
-        unsigned w = 0;
-        {
+            const int sb = lane & 7;
+            const int x = bx + (sb & 1) * (kBrickX / 2), y = by + (sb >> 1 & 1) * (kBrickY / 2),
+                      z = bz + (sb >> 2) * (kBrickZ / 2);
             int n = 0;
-            // (a few bricks go to their sub-bricks at once)
-            if (lane < nb && va.per_claim > 4) n = settle_cells<SQ, MOD, AXIS>(fd, va, step, bx, by, bz, kBrickX, kBrickY, kBrickZ);
+            if ((lane >> 3) < nb && x < g && y < g && z < g) n = settle_cells<SQ, MOD, AXIS>(fd, va, step, x, y, z);
             __syncwarp();
-            w = (unsigned)n * 0x11111111u;
-            unsigned todo = __ballot_sync(kFull, lane < nb && n == 0);
-            while (todo) {
-                int blk = -1, src = -1;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const int bj = todo ? __ffs(todo) - 1 : -1;
-                    todo &= todo - 1;
-                    if ((lane >> 3) == j) blk = bj;
-                    if (lane == bj) src = 8 * j;
-                }
-                const int from = blk < 0 ? 0 : blk, sb = lane & 7;
-                const int x = __shfl_sync(kFull, bx, from) + (sb & 1) * (kBrickX / 2);
-                const int y = __shfl_sync(kFull, by, from) + (sb >> 1 & 1) * (kBrickY / 2);
-                const int z = __shfl_sync(kFull, bz, from) + (sb >> 2) * (kBrickZ / 2);
-                int m = 0;
-                if (blk >= 0 && x < g && y < g && z < g)
-                    m = settle_cells<SQ, MOD, AXIS>(fd, va, step, x, y, z, kBrickX / 2, kBrickY / 2, kBrickZ / 2);
-                __syncwarp();
-                unsigned v = (unsigned)m << (4 * sb);
-                v |= __shfl_xor_sync(kFull, v, 1);
-                v |= __shfl_xor_sync(kFull, v, 2);
-                v |= __shfl_xor_sync(kFull, v, 4);
-                const unsigned t = __shfl_sync(kFull, v, src < 0 ? 0 : src);
-                if (src >= 0) w = t;
-            }
+            w = (unsigned)n << (4 * sb);
+            w |= __shfl_xor_sync(kFull, w, 1);
+            w |= __shfl_xor_sync(kFull, w, 2);
+            w |= __shfl_xor_sync(kFull, w, 4);
         }
         uint32_t it32 = 0, in32 = 0, cl32 = 0, re32 = 0;
         for (int b = 0; b < nb; ++b) {
-            const unsigned word = __shfl_sync(kFull, w, b);
-            const int x0 = __shfl_sync(kFull, bx, b), y0 = __shfl_sync(kFull, by, b), z0 = __shfl_sync(kFull, bz, b);
+            const unsigned word = __shfl_sync(kFull, w, 8 * b);
+            const int x0 = __shfl_sync(kFull, bx, 8 * b), y0 = __shfl_sync(kFull, by, 8 * b),
+                      z0 = __shfl_sync(kFull, bz, 8 * b);
             const int n0 = (int)(word & 15u);
             if (va.wide && n0 && word == (unsigned)n0 * 0x11111111u && x0 + kBrickX <= g) {
                 // a settled brick: 32 rows of 16 cells, one per lane
@@ -496,20 +479,16 @@ cudaError_t launch_voxels_t(const FrameDesc &fd, const VoxelArgs &args, cudaStre
     const bool re = fd.precision == DQJ_FP32_RECHECK;
     const int axis = fd.axis_slice ? 1 : 0;
     if (args.g >= kBrickGrid && fd.blocks) {
-        // bricks per claim: 32 or 16 (one settle pass of a warp) where every resident
-        // warp gets several claims of that, else four (one pass over their sub-bricks)
-        VoxelArgs va = args;
-        const uint32_t warps =
-            (uint32_t)num_sms * (uint32_t)resident_per_sm(gb, voxel_brick_kernel<SQ, MOD, false, false>) * 4u;
-        va.per_claim = va.nbricks >= 256u * warps ? 32u : va.nbricks >= 64u * warps ? 16u : 4u;
-        const uint32_t claims = (va.nbricks + va.per_claim - 1u) / va.per_claim;
-        const int gg = (int)std::min(warps / 4u, (claims + 3u) / 4u);
+        const uint32_t cap =
+            (uint32_t)num_sms * (uint32_t)resident_per_sm(gb, voxel_brick_kernel<SQ, MOD, false, false>);
+        const uint32_t claims = (args.nbricks + kBrickClaim - 1u) / kBrickClaim;
+        const int gg = (int)std::min(cap, (claims + 3u) / 4u);
         if (re)
-            axis ? voxel_brick_kernel<SQ, MOD, true, true><<<gg, kBlock, 0, st>>>(fd, va)
-                 : voxel_brick_kernel<SQ, MOD, true, false><<<gg, kBlock, 0, st>>>(fd, va);
+            axis ? voxel_brick_kernel<SQ, MOD, true, true><<<gg, kBlock, 0, st>>>(fd, args)
+                 : voxel_brick_kernel<SQ, MOD, true, false><<<gg, kBlock, 0, st>>>(fd, args);
         else
-            axis ? voxel_brick_kernel<SQ, MOD, false, true><<<gg, kBlock, 0, st>>>(fd, va)
-                 : voxel_brick_kernel<SQ, MOD, false, false><<<gg, kBlock, 0, st>>>(fd, va);
+            axis ? voxel_brick_kernel<SQ, MOD, false, true><<<gg, kBlock, 0, st>>>(fd, args)
+                 : voxel_brick_kernel<SQ, MOD, false, false><<<gg, kBlock, 0, st>>>(fd, args);
     } else {
         const int gm = (int)min((uint64_t)num_sms * resident_per_sm(g2, voxel2_kernel<SQ, MOD, false, false>),
                                 (args.nsegs + 4 * kBatch - 1) / (4 * kBatch));
