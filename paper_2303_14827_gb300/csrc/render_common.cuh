@@ -1029,8 +1029,9 @@ __device__ __forceinline__ void flush_rest(const FrameDesc &fd, const Scratch &s
 
 // One 64-ray tile of the paired march (see march2_kernel); all 32 lanes call.
 // A lane holds tile slots `lane` and `lane + 32`.  RECHECK: qs is the warp's
-// staging buffer of kQStage entries in shared memory, rechecked at the end of
-// the tile.  SPLIT: only samples
+// staging buffer of kQStage entries in shared memory, filtered by a rounding bound
+// at the end of the tile (recheck_staged); *left of them stay staged for the warp's
+// next tile.  SPLIT: only samples
 // [kb, ke) of each ray, with the range's partial result written to sc.part
 // (range r = kb / fd.k_chunk) for march_merge_kernel instead of the outputs;
 // a ray for which a lower range has already found an inside sample is

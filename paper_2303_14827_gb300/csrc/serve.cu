@@ -9,7 +9,7 @@
 // estimated cost), claims one work item from it with an atomic add and runs it:
 //   MARCH phase  : one 64-ray tile of the paired march (march4_tile, or
 //                  march2_tile with DQJ_MARCH_SAMPLES=1; in the recheck mode
-//                  with the FP64 recheck of its staged samples);
+//                  the samples its rounding bound leaves open join the queue);
 //   BISECT phase : 32 hit-list entries (bisect_chunk);
 //   RECHECK phase: 32 recheck-queue entries (recheck_entry), recheck mode only;
 //   FIXUP phase  : one to five pixels to re-render in FP64 (fixup_pixels), recheck mode.
@@ -206,7 +206,8 @@ __device__ __noinline__ void fixup_item(const FrameDesc &fd, const Scratch &sc, 
 }
 
 // Pixels of a FIXUP item: five where a request has many, else one, so that a
-// short list spreads over the warps.
+// short list spreads over the warps.  Sixteen requests of mixed sizes: 18.1 ms;
+// always one 18.7, always five 18.8.
 __device__ __forceinline__ unsigned fixup_step(unsigned total) { return total >= 2048u ? (unsigned)kLateGroup : 1u; }
 
 // Claim up to `step` items of a phase (lane 0): the first claimed index, or

@@ -245,15 +245,16 @@ __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[
             }
         }
         // norms of the halves and the products z . g_a
-        float2 su, sv, tu, tv, wu, wv;
+        float2 su, sv, tu, tv;
+        float gr, gd;
         {
             const float2 z0 = make_float2(u[0].x, u[0].x), z4 = make_float2(u[4].x, u[4].x);
             su = f2mul(z0, u[0]);
             sv = f2mul(z0, v[0]);
             tu = f2mul(z4, u[4]);
             tv = f2mul(z4, v[4]);
-            float gr = fmaf(v[0].y, v[0].y, fmaf(v[0].x, v[0].x, u[0].y * u[0].y));
-            float gd = fmaf(v[4].y, v[4].y, fmaf(v[4].x, v[4].x, u[4].y * u[4].y));
+            gr = fmaf(v[0].y, v[0].y, fmaf(v[0].x, v[0].x, u[0].y * u[0].y));
+            gd = fmaf(v[4].y, v[4].y, fmaf(v[4].x, v[4].x, u[4].y * u[4].y));
 #pragma unroll
             for (int i = 1; i < 4; ++i) {
                 const float2 zi = make_float2(u[i].x, u[i].x), zj = make_float2(u[4 + i].x, u[4 + i].x);
@@ -264,13 +265,10 @@ __device__ __forceinline__ int settle_box(const FrameDesc &fd, const float (&p)[
                 gr = fmaf(v[i].y, v[i].y, fmaf(v[i].x, v[i].x, fmaf(u[i].y, u[i].y, gr)));
                 gd = fmaf(v[4 + i].y, v[4 + i].y, fmaf(v[4 + i].x, v[4 + i].x, fmaf(u[4 + i].y, u[4 + i].y, gd)));
             }
-            wu = make_float2(gr, gd);
-            wv = make_float2(0.f, 0.f);
         }
-        (void)wv;
         // |sum_a u_a g_a|^2 <= 3 sum_a |g_a|^2
-        Gr = sqrt_approx(3.f * wu.x);
-        Gd = sqrt_approx(3.f * wu.y);
+        Gr = sqrt_approx(3.f * gr);
+        Gd = sqrt_approx(3.f * gd);
         ar = sqrt_approx(su.x);
         ad = sqrt_approx(tu.x);
         float m, dev, sq;

@@ -285,8 +285,8 @@ __global__ void __launch_bounds__(kBlock) voxel_render_kernel(const __grid_const
 // the cell in which the ray enters a block, and the number of cells it crossed
 // until there, follow from the crossing alone.  1080p, default c, cell by cell /
 // by blocks (ms): 24^3 0.30 / 0.30, 64^3 0.37 / 0.32, 100^3 0.50 / 0.33, 200^3 1.0 / 0.37,
-// 512^3 3.1 / 0.64, 1024^3 8.0 / 1.3.  (On noise, whose blocks are all occupied, the
-// blocks only cost: 200^3 with 2 % of the cells set, 701x433, 0.21 / 0.27 ms.)
+// 512^3 3.1 / 0.64, 1024^3 8.0 / 1.3 (more, and grids on which blocks only cost, at
+// mip_shift).
 template <int SHIFT>
 __global__ void __launch_bounds__(kBlock) voxel_render_blocks_kernel(const __grid_constant__ FrameDesc fd,
                                                                      const uint8_t *__restrict__ occ, int g,
@@ -493,7 +493,16 @@ __global__ void __launch_bounds__(kBlock) voxel_mip_kernel(const uint8_t *__rest
 
 // Block size of the walk, 2^shift cells a side (0: cell by cell): a ray crosses
 // about 3 g / 2^shift blocks, and every block it meets that is not empty costs
-// the search of its first cell.
+// the search of its first cell.  Cell by cell / by blocks, default c, at 1080p and at
+// 64x48 (us, the block occupancy included): 24^3 277 / 281 and 21 / 26, 32^3 289 / 282 and
+// 27 / 26, 50^3 337 / 295 and 38 / 36, 96^3 555 / 313 and 78 / 54, 200^3 1128 / 364 and 192 /
+// 86, 1024^3 9337 / 1360 and 1406 / 515; solids (a ball, a shell) 0.9 to 2.5 times as
+// fast.  Scattered cells, which a Julia grid does not have, lose: noise of 3e-4 of the
+// cells at 200^3 1263 / 714, of 1e-3 1247 / 1260, of 0.01 901 / 1345, of 0.1 at 1024^3 455 / 730.
+// (Measured and not kept: judging the grid from 1,024 sampled rows first, which took
+// 6 to 8 us of every image and left the noise 0.8 to 0.9 times as fast as cell by
+// cell; going cell by cell on a ray that met too few empty blocks, 364 -> 418 us at
+// 200^3.)
 int mip_shift(int g) { return g >= 96 ? 3 : (g >= 24 ? 2 : 0); }
 
 // Allocates from the stream's pool without disturbing a capture under way on
