@@ -70,6 +70,15 @@ __global__ void sample_kernel(const __grid_constant__ FrameDesc fd, const int *x
     wrong[i] = count_certain<SQ, MOD, AXIS>(fd, x[i], y[i], k[i], c + 1);
 }
 
+// The integer doublings: 2 x and 4 x of every bit pattern.
+__global__ void twice_kernel(const double *x, long n, double *two, double *four)
+{
+    const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    two[i] = twice(x[i]);
+    four[i] = four_times(x[i]);
+}
+
 // One warp: n staged entries of march samples whose FP32 count is wrong by one,
 // against a queue of `cap` entries; ctr, flags and list as in a frame's scratch.
 __global__ void staged_kernel(const __grid_constant__ FrameDesc fd, Scratch sc, const int4 *entries, int n)
@@ -180,6 +189,12 @@ int probe_samples(const dqj_params *p, const int *x, const int *y, const int *k,
     case 2: run(O{}, Z{}); break;
     default: run(O{}, O{}); break;
     }
+    return done();
+}
+
+int probe_twice(const double *x, long n, double *two, double *four)
+{
+    twice_kernel<<<(unsigned)((n + 127) / 128), 128>>>(x, n, two, four);
     return done();
 }
 

@@ -1,8 +1,8 @@
 """The recheck's device functions against plain FP64, called one by one through a
 probe library built from the same headers (bounds_probe.cu): the FP64 clip of a
 ray, the positions of samples, the two orbit bounds, the bound of a march
-sample's position, and what becomes of staged samples that find the recheck queue
-full."""
+sample's position, the FP64 doublings on the integer units, and what becomes of
+staged samples that find the recheck queue full."""
 import ctypes
 import os
 import subprocess
@@ -175,6 +175,24 @@ def test_orbit_bounds(probe, square, modulus, radius):
                 decided[which] += int(certain.sum())
             assert np.array_equal(classify(probe, p, 3, pts)[0], want)
     assert decided[0] > 0.2 * 48 * n and decided[1] > decided[0]  # the bounds decide something
+
+
+def test_integer_doubling(probe):
+    # every exponent and sign: zeros, subnormals (whose carry enters the exponent),
+    # normals, overflow, infinities and NaN
+    import torch
+    edges = np.array([0, 1, 2, 0x80000000, 0xffffffff, 1 << 32, (1 << 51) - 1, 1 << 51, (1 << 52) - 1], dtype=np.uint64)
+    m = np.concatenate([edges, np.random.default_rng(5).integers(0, 1 << 52, 500, dtype=np.uint64)])
+    bits = ((np.arange(4096, dtype=np.uint64) << np.uint64(52))[:, None] | m[None]).ravel()
+    x = dev(bits.view(np.float64))
+    out = torch.empty(2, x.numel(), dtype=torch.float64, device="cuda")
+    assert probe.probe_twice(ptr(x), ctypes.c_long(x.numel()), ptr(out[0]), ptr(out[1])) == 0
+    with np.errstate(all="ignore"):
+        want = bits.view(np.float64) * 2.0, bits.view(np.float64) * 4.0
+    for got, w in zip(out.cpu().numpy(), want):
+        nan = np.isnan(w)
+        assert np.array_equal(np.isnan(got), nan)
+        assert np.array_equal(got[~nan].view(np.uint64), w[~nan].view(np.uint64))
 
 
 VIEWS = (dict(), dict(eye=[2.0001, 2.0001, 2.00013]), dict(eye=[0.3, 1.999, 0.2]), dict(eye=[1.1, 0.4, 0.9]),

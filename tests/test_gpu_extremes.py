@@ -1,12 +1,12 @@
 """Calls at the ends of what the parameters allow: boxes whose samples overflow,
-escape radii below what FP32 squares resolve, and rays that run almost parallel
-to a slab they lie outside of."""
+escape radii below what FP32 squares resolve, rays that run almost parallel
+to a slab they lie outside of, and eyes beside the box's faces and corners."""
 import numpy as np
 import pytest
 
 import oracle
 from paper_2303_14827_gb300 import binding, scenes
-from parity import to_numpy
+from parity import assert_parity, compare, to_numpy
 
 pytestmark = pytest.mark.gpu
 
@@ -69,3 +69,16 @@ def test_voxel_ray_beside_the_grid(g, side):
         torch.cuda.synchronize()
         out = to_numpy(t, 64, 1)
     assert np.all(np.isinf(out["depth"])) and np.all(out["iter"] == 0)
+
+
+@pytest.mark.parametrize("precision", (1, 2))
+@pytest.mark.parametrize("off", (1e-3, 1e-4, 1e-6, -1e-3, -1e-6))
+@pytest.mark.parametrize("sides", [(1, 1, 1.3), (0, 1, 0), (1, 0, 1.7), (-1, -1, -1)])
+def test_eye_beside_the_box(sides, off, precision):
+    # off > 0 outside, < 0 inside; 0 in sides: well inside the slab
+    eye = [2.0 * np.sign(d) + off * d if d else 0.31 for d in sides]
+    s = scenes.default_scene(width=96, height=72, precision=precision, eye=eye, target=[0.05, -0.11, 0.02],
+                             fov_y_deg=60.0, march_steps=400, bisect_steps=8, max_iter=16)
+    with binding.Renderer(0) as r:
+        g = to_numpy(r.render(s), 96, 72)
+    assert_parity(compare(g, oracle.render(s)), what=f"eye {eye}")
